@@ -22,6 +22,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -291,60 +292,152 @@ __global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, siz
 }
 
 // ------------------------------------------------------------------- gamma
-__device__ __forceinline__ float trilinear(const float* __restrict__ f, int nx, int ny, int nz, float px, float py,
-                                           float pz) {
-    px = fminf(fmaxf(px, 0.f), (float)(nx - 1));
-    py = fminf(fmaxf(py, 0.f), (float)(ny - 1));
-    pz = fminf(fmaxf(pz, 0.f), (float)(nz - 1));
-    const int x0 = min((int)px, max(nx - 2, 0)), y0 = min((int)py, max(ny - 2, 0)), z0 = min((int)pz, max(nz - 2, 0));
-    const int x1 = min(x0 + 1, nx - 1), y1 = min(y0 + 1, ny - 1), z1 = min(z0 + 1, nz - 1);
-    const float fx = px - x0, fy = py - y0, fz = pz - z0;
-    auto at = [&](int x, int y, int z) { return f[((size_t)z * ny + y) * nx + x]; };
-    const float c00 = at(x0, y0, z0) * (1 - fx) + at(x1, y0, z0) * fx;
-    const float c10 = at(x0, y1, z0) * (1 - fx) + at(x1, y1, z0) * fx;
-    const float c01 = at(x0, y0, z1) * (1 - fx) + at(x1, y0, z1) * fx;
-    const float c11 = at(x0, y1, z1) * (1 - fx) + at(x1, y1, z1) * fx;
-    return (c00 * (1 - fy) + c10 * fy) * (1 - fz) + (c01 * (1 - fy) + c11 * fy) * fz;
+// One axis of a trilinear lookup at coordinate p (voxel units, clamped to the grid of n).
+struct Lerp {
+    int i0, i1;
+    float f;
+};
+__device__ __forceinline__ Lerp lerp_at(float p, int n) {
+    p = fminf(fmaxf(p, 0.f), (float)(n - 1));
+    Lerp l;
+    l.i0 = min((int)p, max(n - 2, 0));
+    l.i1 = min(l.i0 + 1, n - 1);
+    l.f = p - l.i0;
+    return l;
 }
 
-// Local-normalisation gamma: a reference voxel with dose >= thr passes when some
+constexpr int kGammaMaxSteps = 50;
+constexpr int kGammaChunk = 128;  // voxels a block claims at a time
+struct GammaCtl {
+    unsigned long long evaluated, passed, cursor;
+    unsigned int maxbits, pad;
+};
+
+// Local-normalisation gamma: a reference voxel with dose >= threshold max(ref) passes when some
 // evaluated position within the DTA ball (grid step dta/steps, trilinear) has
-// |dr|^2/dta^2 + (De - Dr)^2/(dd Dr)^2 <= 1.  counts[0] += evaluated, counts[1] += passed.
-__global__ void k_gamma(const float* __restrict__ ref, const float* __restrict__ ev, int nx, int ny, int nz, float hx,
-                        float hy, float hz, float dd, float dta, float thr, int steps, unsigned long long* counts) {
+// |dr|^2/dta^2 + (De - Dr)^2/(dd Dr)^2 <= 1.  ctl counts the evaluated and the passing voxels.
+//
+// Most voxels are below the threshold or pass at their own position; the search over the ball
+// (9261 positions at 10 steps) runs only for the rest, which are few and clustered.  So blocks
+// claim chunks of 128 voxels from a cursor, test them one per thread, list those that need the
+// search in shared memory, and each warp then searches one voxel with a lane per (y, x)
+// offset of the disk: the lanes walk the z offsets together, interpolate a plane in x and y only
+// when z crosses into the next voxel, skip the offsets between two planes where no lane's dose
+// can come within the tolerance, and stop as soon as a lane passes.  Bound by instruction
+// issue of that walk.  192x128x128, 2 %/0.5 mm, 10 steps: 10.7 ms with one lane per voxel
+// walking the whole ball, 0.42 ms so.
+__global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, const float* __restrict__ ev, int nx,
+                                               int ny, int nz, float hx, float hy, float hz, float dd, float dta,
+                                               double threshold, int steps, GammaCtl* ctl) {
+    __shared__ float s_q[3][2 * kGammaMaxSteps + 1];                     // offset a st / h per axis
+    __shared__ char2 s_yx[(2 * kGammaMaxSteps + 1) * (2 * kGammaMaxSteps + 1)];  // (y, x) offsets in the disk
+    __shared__ float4 s_z[8][2 * kGammaMaxSteps + 1];  // per warp: z offset, its fraction f, 1 - f, voxel
+    __shared__ int s_npairs, s_nlist;
+    __shared__ unsigned long long s_claim;
+    __shared__ unsigned char s_list[kGammaChunk];
     const size_t n = (size_t)nx * ny * nz;
-    unsigned int evals = 0, passes = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float r = ref[i];
-        if (!(r >= thr) || !(r > 0.f)) continue;
-        evals += 1;
-        const float tol = dd * r;
-        bool pass = fabsf(ev[i] - r) <= tol;
-        if (!pass) {
-            const int ix = (int)(i % nx), iy = (int)((i / nx) % ny), iz = (int)(i / ((size_t)nx * ny));
-            const float st = dta / steps, inv_dta2 = 1.f / (dta * dta), inv_tol2 = 1.f / (tol * tol);
-            for (int a = -steps; a <= steps && !pass; ++a)
-                for (int b = -steps; b <= steps && !pass; ++b)
-                    for (int c = -steps; c <= steps; ++c) {
-                        const float oz = a * st, oy = b * st, ox = c * st;
-                        const float d2 = (ox * ox + oy * oy + oz * oz) * inv_dta2;
-                        if (d2 > 1.f) continue;
-                        const float e = trilinear(ev, nx, ny, nz, ix + ox / hx, iy + oy / hy, iz + oz / hz);
-                        if (d2 + (e - r) * (e - r) * inv_tol2 <= 1.f) {
-                            pass = true;
-                            break;
-                        }
-                    }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, side = 2 * steps + 1;
+    const float st = dta / steps, inv_dta2 = 1.f / (dta * dta);
+    const float thr = (float)(threshold * (double)__uint_as_float(ctl->maxbits));
+    for (int i = tid; i < side; i += blockDim.x) {
+        const float o = (i - steps) * st;
+        s_q[0][i] = o / hx;
+        s_q[1][i] = o / hy;
+        s_q[2][i] = o / hz;
+    }
+    if (warp == 0) {  // rows of the disk in the order 0, 1, -1, 2, -2 ...: a pass is usually found near 0
+        int at = 0;
+        for (int p0 = 0; p0 < side * side; p0 += 32) {
+            const int p = p0 + lane, r = p / side;
+            const int b = (r & 1) ? (r + 1) / 2 : -(r / 2), c = p - r * side - steps;
+            const float oy = b * st, ox = c * st;
+            const bool in = p < side * side && (ox * ox + oy * oy) * inv_dta2 <= 1.f;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (in) s_yx[at + __popc(m & ((1u << lane) - 1u))] = make_char2((signed char)b, (signed char)c);
+            at += __popc(m);
         }
-        passes += pass ? 1u : 0u;
+        if (lane == 0) s_npairs = at;
+    }
+    unsigned int evals = 0, passes = 0;
+    for (;;) {
+        __syncthreads();  // the list and the claim of the previous round are no longer read
+        if (tid == 0) {
+            s_claim = atomicAdd(&ctl->cursor, (unsigned long long)kGammaChunk);
+            s_nlist = 0;
+        }
+        __syncthreads();
+        const size_t base = (size_t)s_claim;
+        if (base >= n) break;
+        if (tid < kGammaChunk && base + tid < n) {
+            const float r = ref[base + tid];
+            if (r >= thr && r > 0.f) {
+                evals += 1;
+                if (fabsf(ev[base + tid] - r) <= dd * r)
+                    passes += 1;
+                else
+                    s_list[atomicAdd(&s_nlist, 1)] = (unsigned char)tid;
+            }
+        }
+        __syncthreads();
+        const int nlist = s_nlist, npairs = s_npairs;
+        for (int j = warp; j < nlist; j += 8) {
+            const size_t i = base + s_list[j];
+            const float r = ref[i];
+            const float tol = dd * r, inv_tol2 = 1.f / (tol * tol);
+            const int ix = (int)(i % nx), iy = (int)((i / nx) % ny), iz = (int)(i / ((size_t)nx * ny));
+            __syncwarp();
+            for (int k = lane; k < side; k += 32) {  // the walk along z is the same for every lane
+                const Lerp z = lerp_at(iz + s_q[2][k], nz);
+                s_z[warp][k] = make_float4((k - steps) * st, z.f, 1 - z.f, __int_as_float(z.i0));
+            }
+            __syncwarp();
+            const float reach = tol * 1.00001f;  // no rounding of the test below passes beyond this
+            bool pass = false;
+            for (int p0 = 0; p0 < npairs; p0 += 32) {
+                const bool have = p0 + lane < npairs;
+                const char2 yx = s_yx[have ? p0 + lane : 0];
+                const float oy = yx.x * st, ox = yx.y * st;
+                const Lerp x = lerp_at(ix + s_q[0][yx.y + steps], nx), y = lerp_at(iy + s_q[1][yx.x + steps], ny);
+                const float* f0 = ev + (size_t)y.i0 * nx;
+                const float* f1 = ev + (size_t)y.i1 * nx;
+                auto plane = [&](int z) {
+                    const size_t o = (size_t)z * ny * nx;
+                    const float c0 = f0[o + x.i0] * (1 - x.f) + f0[o + x.i1] * x.f;
+                    const float c1 = f1[o + x.i0] * (1 - x.f) + f1[o + x.i1] * x.f;
+                    return c0 * (1 - y.f) + c1 * y.f;
+                };
+                int zc = -2;
+                float lo = 0.f, hi = 0.f;
+                bool cell = false;  // some lane's dose between the two planes may come near r
+                for (int k = 0; k < side; ++k) {
+                    const float4 q = s_z[warp][k];
+                    const int z0 = __float_as_int(q.w);
+                    if (z0 != zc) {
+                        lo = z0 == zc + 1 ? hi : plane(z0);
+                        hi = plane(min(z0 + 1, nz - 1));
+                        zc = z0;
+                        const float slack = reach + 1e-6f * fmaxf(fmaxf(fabsf(lo), fabsf(hi)), r);
+                        cell = __any_sync(0xffffffffu, !(fmaxf(lo, hi) < r - slack) && !(fminf(lo, hi) > r + slack));
+                    }
+                    if (!cell) continue;
+                    const float d2 = (ox * ox + oy * oy + q.x * q.x) * inv_dta2;
+                    const float e = lo * q.z + hi * q.y;
+                    pass |= d2 <= 1.f && d2 + (e - r) * (e - r) * inv_tol2 <= 1.f;
+                }
+                if (__any_sync(0xffffffffu, pass && have)) {
+                    passes += lane == 0 ? 1u : 0u;
+                    break;
+                }
+            }
+        }
     }
     for (int off = 16; off > 0; off >>= 1) {
         evals += __shfl_down_sync(0xffffffffu, evals, off);
         passes += __shfl_down_sync(0xffffffffu, passes, off);
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&counts[0], (unsigned long long)evals);
-        atomicAdd(&counts[1], (unsigned long long)passes);
+    if (lane == 0) {
+        if (evals) atomicAdd(&ctl->evaluated, (unsigned long long)evals);
+        if (passes) atomicAdd(&ctl->passed, (unsigned long long)passes);
     }
 }
 
@@ -402,8 +495,6 @@ struct sde_denoiser {
         *g_e1a;
     unsigned int* maxbits;
     float* loss_acc;
-    unsigned long long* gcounts;
-    unsigned int* gmax;
 };
 
 namespace {
@@ -592,6 +683,59 @@ int backward(sde_denoiser* d, int batch) {
     return fail(cudaGetLastError(), "backward launch");
 }
 
+// A counter block for one gamma call.  The call waits for its work, so blocks can be handed
+// out and taken back on the host: 64 per device, allocated once (an allocation per call cost
+// ~120 us after every wait, when the stream-ordered pool has given its memory back); a 65th
+// concurrent call allocates its own.
+struct GammaSlot {
+    static constexpr int kSlots = 64, kDevices = 64;
+    GammaCtl* ctl = nullptr;
+    int dev = -1, index = -1;
+
+    struct Shared {
+        std::mutex m;
+        GammaCtl* base[kDevices] = {};
+        uint64_t busy[kDevices] = {};
+    };
+    static Shared& shared() {
+        static Shared* s = new Shared();  // never destroyed: calls may come from exit handlers
+        return *s;
+    }
+    int take(cudaStream_t st) {
+        DN_TRY(fail(cudaGetDevice(&dev), "cudaGetDevice"));
+        Shared& s = shared();
+        if (dev >= 0 && dev < kDevices) {
+            std::lock_guard<std::mutex> lock(s.m);
+            if (!s.base[dev]) {
+                void* p = nullptr;
+                cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // another thread may be capturing
+                cudaThreadExchangeStreamCaptureMode(&mode);
+                const cudaError_t e = cudaMalloc(&p, kSlots * sizeof(GammaCtl));
+                cudaThreadExchangeStreamCaptureMode(&mode);
+                DN_TRY(fail(e, "cudaMalloc"));
+                s.base[dev] = static_cast<GammaCtl*>(p);
+            }
+            for (int i = 0; i < kSlots; ++i)
+                if (!(s.busy[dev] >> i & 1)) {
+                    s.busy[dev] |= 1ull << i;
+                    index = i;
+                    ctl = s.base[dev] + i;
+                    return SDE_OK;
+                }
+        }
+        return fail(cudaMallocAsync(reinterpret_cast<void**>(&ctl), sizeof(GammaCtl), st), "alloc");
+    }
+    void release(cudaStream_t st) {  // after the call's work has been waited for
+        if (index < 0) {
+            cudaFreeAsync(ctl, st);
+            return;
+        }
+        Shared& s = shared();
+        std::lock_guard<std::mutex> lock(s.m);
+        s.busy[dev] &= ~(1ull << index);
+    }
+};
+
 // After every change of the BF16 weights: the flipped copies and both packed images.
 int refresh_weights(sde_denoiser* d) {
     for (int i = 0; i < 11; ++i) {
@@ -698,8 +842,6 @@ extern "C" int sde_denoiser_create(sde_denoiser** out, int D, int H, int W, int 
     if (!rc) rc = dalloc(d, &d->out, d->V1 * B);  // FP32 output channel 0, plain [n][voxel]
     if (!rc) rc = dalloc(d, &d->maxbits, B);
     if (!rc) rc = dalloc(d, &d->loss_acc, (size_t)1);
-    if (!rc) rc = dalloc(d, &d->gcounts, (size_t)2);
-    if (!rc) rc = dalloc(d, &d->gmax, (size_t)1);
     if (!rc) rc = refresh_weights(d);
     if (!rc) rc = fail(cudaDeviceSynchronize(), "create sync");
     if (rc) {
@@ -870,37 +1012,27 @@ extern "C" int sde_gamma3d(const float* d_ref, const float* d_eval, int nx, int 
                            double dd, double dta_mm, double threshold, int steps, uint64_t* n_eval,
                            uint64_t* n_pass, void* stream) {
     if (!d_ref || !d_eval || nx < 1 || ny < 1 || nz < 1 || !voxel_mm || !(dd > 0) || !(dta_mm > 0) || steps < 1 ||
-        steps > 50 || !n_eval || !n_pass) {
+        steps > kGammaMaxSteps || !n_eval || !n_pass) {
         set_last_error("sde_gamma3d: bad arguments");
         return SDE_EINVAL;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    unsigned long long* counts = nullptr;
-    unsigned int* mx = nullptr;
-    DN_TRY(fail(cudaMallocAsync(&counts, 2 * sizeof(unsigned long long) + sizeof(unsigned int), st), "alloc"));
-    mx = reinterpret_cast<unsigned int*>(counts + 2);
-    int rc = fail(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long) + sizeof(unsigned int), st), "memset");
+    GammaSlot slot;
+    DN_TRY(slot.take(st));
     const size_t n = (size_t)nx * ny * nz;
-    unsigned int h_mx = 0;
-    unsigned long long h[2] = {0, 0};
+    GammaCtl h{};
+    int rc = fail(cudaMemsetAsync(slot.ctl, 0, sizeof(GammaCtl), st), "memset");
     if (!rc) {
-        k_max<<<kBlocks, 256, 0, st>>>(d_ref, n, mx);
-        rc = fail(cudaMemcpyAsync(&h_mx, mx, sizeof h_mx, cudaMemcpyDeviceToHost, st), "copy");
-    }
-    if (!rc) rc = fail(cudaStreamSynchronize(st), "sync");
-    if (!rc) {
-        float dmax;
-        memcpy(&dmax, &h_mx, sizeof dmax);
+        k_max<<<kBlocks, 256, 0, st>>>(d_ref, n, &slot.ctl->maxbits);
         k_gamma<<<kBlocks, 256, 0, st>>>(d_ref, d_eval, nx, ny, nz, (float)voxel_mm[0], (float)voxel_mm[1],
-                                         (float)voxel_mm[2], (float)dd, (float)dta_mm, (float)(threshold * dmax),
-                                         steps, counts);
+                                         (float)voxel_mm[2], (float)dd, (float)dta_mm, threshold, steps, slot.ctl);
         rc = fail(cudaGetLastError(), "gamma launch");
     }
-    if (!rc) rc = fail(cudaMemcpyAsync(h, counts, sizeof h, cudaMemcpyDeviceToHost, st), "copy");
-    if (!rc) rc = fail(cudaStreamSynchronize(st), "sync");
-    cudaFreeAsync(counts, st);
-    if (rc) return rc;
-    *n_eval = h[0];
-    *n_pass = h[1];
+    if (!rc) rc = fail(cudaMemcpyAsync(&h, slot.ctl, sizeof h, cudaMemcpyDeviceToHost, st), "copy");
+    const int rs = fail(cudaStreamSynchronize(st), "sync");
+    slot.release(st);
+    if (rc || rs) return rc ? rc : rs;
+    *n_eval = h.evaluated;
+    *n_pass = h.passed;
     return SDE_OK;
 }
