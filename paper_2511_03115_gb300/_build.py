@@ -17,10 +17,16 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUTDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUTDIR, "libsde_dose.so")
-SOURCES = ["sde_api.cu", "sde_tables.cu", "sde_transport.cu", "sde_noalloc.cu", "sde_denoise.cu", "sde_denoiser.cu"]
+SOURCES = ["sde_api.cu", "sde_tables.cu", "sde_transport.cu", "sde_tally.cu", "sde_noalloc.cu", "sde_denoise.cu", "sde_denoiser.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
+
+# The transport kernel flushes subnormal numbers to zero: without it every approximate logarithm,
+# root and reciprocal of the step carries instructions for subnormal arguments, which its
+# energies, random numbers and rates never are (same tallies; slab of 10^6 protons 4.79 -> 4.38 ms,
+# 2000-spot plan of 3 10^7 113.2 -> 105.4 ms).
+FILE_FLAGS = {"sde_transport.cu": ["-ftz=true"]}
 
 
 def nvcc() -> str:
@@ -47,7 +53,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), lib_path: 
 
     def compile_one(src):
         obj = os.path.join(os.path.dirname(lib_path), src.replace(".cu", f".{os.getpid()}.o"))
-        cmd = [cc, *ARCH, *FLAGS, *extra_flags, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [cc, *ARCH, *FLAGS, *FILE_FLAGS.get(src, []), *extra_flags, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")

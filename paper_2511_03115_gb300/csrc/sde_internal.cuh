@@ -160,7 +160,7 @@ __device__ __forceinline__ unsigned long long qfix(const KParams& P, float E) {
 // (measured 4 % of the transport kernel).
 __device__ __forceinline__ float step_sqrt(float x) {
     float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 

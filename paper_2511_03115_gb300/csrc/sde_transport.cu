@@ -83,7 +83,7 @@ __device__ __forceinline__ float cut_rate(const KParams& P, int m, const Phys& p
     float R = fmaf(a.y, ph.f, a.x), Hc = fmaf(a.w, ph.f, a.z), Hlo = fmaf(b.y, ph.f, b.x);
     float rate = R * (__fdividef(1.f, s_c) - 0.5f) - Hlo;
     if (Hc > 0.f) {
-        float eta = (float)kFineStructure * rsqrtf(2.f * E / (float)kProtonMass);
+        float eta = (float)kFineStructure * rsqrtf(__fdiv_rn(2.f * E, (float)kProtonMass));
         rate = fmaf(Hc, mott_prim(s_c, eta), rate);
     }
     return rate * __fdividef(1.f, E * E);
@@ -225,7 +225,7 @@ __device__ __forceinline__ JumpOut do_jump(const KParams& P, int m, float E, int
     const float* r0 = P.jrates + (uint32_t)(m * P.N + k) * (uint32_t)(2 * SDE_MAX_ELEMENTS);
     const float* r1 = r0 + 2 * SDE_MAX_ELEMENTS;
     const float rE2 = __fdividef(1.f, E * E);  // elastic rates are stored times E^2
-    const float eta_h = (float)kFineStructure * rsqrtf(2.f * E / (float)kProtonMass);
+    const float eta_h = (float)kFineStructure * rsqrtf(__fdiv_rn(2.f * E, (float)kProtonMass));
     // The stored elastic rates are those of the fixed cut-off s_cut; with the variable
     // cut-off s_c they scale by the ratio of the angular factors (Rutherford: 1/s - 1/2,
     // hydrogen: G(s) - G(mu_lo)).
@@ -801,82 +801,6 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
 }
 #undef SDE_BLOCK_ADD
 
-// Sum of the tally (the deposited energy of the balance), added to *out.
-__global__ void k_sum_u64(const unsigned long long* __restrict__ v, size_t n, unsigned long long* out) {
-    unsigned long long acc = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        acc += v[i];
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, acc);
-}
-
-// Spot records -> device form and the inclusive prefix of history counts;
-// sets the work-queue cursor to the first history id of the run.  One block.
-__global__ void __launch_bounds__(1024) k_prep_spots(const sde_spot* raw, int n, SpotDev* out,
-                                                     unsigned long long* prefix,
-                                                     unsigned long long* counters, unsigned int* err,
-                                                     double ox, double oy, double oz, double ihx, double ihy,
-                                                     double ihz, double e_min, double e_lim,
-                                                     unsigned long long h_begin) {
-    __shared__ unsigned long long scan[1024];
-    unsigned long long carry = 0;
-    for (int base = 0; base < n; base += blockDim.x) {
-        int i = base + threadIdx.x;
-        unsigned long long nh = 0;
-        if (i < n) {
-            sde_spot s = raw[i];
-            double un = s.ux * s.ux + s.uy * s.uy + s.uz * s.uz;
-            bool ok = s.E_MeV > e_min && s.E_MeV + 5.0 * s.sigma_E_MeV <= e_lim && s.sigma_E_MeV >= 0.0 &&
-                      s.sigma_xy_mm >= 0.0 && s.sigma_xy_mm < 1e4 && s.sigma_angle_rad >= 0.0 &&
-                      s.sigma_angle_rad < 1.0 && un > 0.0 && isfinite(un) && isfinite(s.x_mm) &&
-                      isfinite(s.y_mm) && isfinite(s.z_mm);
-            SpotDev d = {};
-            if (ok) {
-                nh = s.n_hist;
-                double inv = rsqrt(un);
-                double x = s.ux * inv, y = s.uy * inv, z = s.uz * inv;
-                double sg = copysign(1.0, z);
-                double a = -1.0 / (sg + z), b = x * y * a;
-                d.E = (float)s.E_MeV;
-                d.sE = (float)s.sigma_E_MeV;
-                d.sxy = (float)s.sigma_xy_mm;
-                d.sang = (float)s.sigma_angle_rad;
-                const double sx = s.sigma_xy_mm * ihx, sy = s.sigma_xy_mm * ihy, sz = s.sigma_xy_mm * ihz;
-                d.px = (float)((s.x_mm - ox) * ihx);
-                d.py = (float)((s.y_mm - oy) * ihy);
-                d.pz = (float)((s.z_mm - oz) * ihz);
-                d.ux = (float)x;
-                d.uy = (float)y;
-                d.uz = (float)z;
-                d.e1x = (float)((1.0 + sg * x * x * a) * sx);
-                d.e1y = (float)(sg * b * sy);
-                d.e1z = (float)(-sg * x * sz);
-                d.e2x = (float)(b * sx);
-                d.e2y = (float)((sg + y * y * a) * sy);
-                d.e2z = (float)(-y * sz);
-            } else {
-                atomicOr(err, kErrBadSpot);
-            }
-            out[i] = d;
-        }
-        scan[threadIdx.x] = nh;
-        __syncthreads();
-        for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-            unsigned long long add = threadIdx.x >= (unsigned)off ? scan[threadIdx.x - off] : 0ull;
-            __syncthreads();
-            scan[threadIdx.x] += add;
-            __syncthreads();
-        }
-        if (i < n) prefix[i + 1] = carry + scan[threadIdx.x];
-        carry += scan[blockDim.x - 1];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        prefix[0] = 0;
-        counters[kCntCursor] = h_begin;
-    }
-}
-
 __global__ void k_probe(const __grid_constant__ KParams P, int m, float rho, float E0, uint64_t h0, int n, float* Eo, float* co,
                         int* jo, float* uxo, float* uyo) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -893,25 +817,6 @@ __global__ void k_probe(const __grid_constant__ KParams P, int m, float rho, flo
     jo[i] = j;
     uxo[i] = ux;
     uyo[i] = uy;
-}
-
-// Dose to medium (Sec. 2.2.2): tally units -> J over voxel mass (kg).  The FP64 unit of
-// this GPU is narrow and a double division is a long sequence on it, so 1/mass is the
-// FP32 reciprocal refined by one Newton step in FP64 (relative error ~1e-14).
-template <typename T>
-__global__ void k_convert(const unsigned long long* edep, const float* rho, size_t nv, double unit_J,
-                          double vol_kg_per_rho, T* dose) {
-    for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nv; v += (size_t)gridDim.x * blockDim.x) {
-        const float r = rho[v];
-        double out = 0.0;
-        if (r > 0.f) {
-            const double mass = (double)r * vol_kg_per_rho;
-            double y = (double)__frcp_rn(__double2float_rn(mass));
-            y = fma(y, fma(-mass, y, 1.0), y);
-            out = (double)edep[v] * unit_J * y;
-        }
-        dose[v] = (T)out;
-    }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -1024,38 +929,10 @@ cudaError_t launch_branch_chunk(unsigned long long* counters, unsigned long long
     return cudaGetLastError();
 }
 
-cudaError_t launch_prep(const sde_spot* raw, int n, SpotDev* out, unsigned long long* prefix,
-                        unsigned long long* counters, unsigned int* err, const double o[3], const double h[3],
-                        double e_min, double e_lim, cudaStream_t st, unsigned long long h_begin) {
-    k_prep_spots<<<1, 1024, 0, st>>>(raw, n, out, prefix, counters, err, o[0], o[1], o[2], 1.0 / h[0], 1.0 / h[1],
-                                     1.0 / h[2], e_min, e_lim, h_begin);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_probe(const KParams& P, int m, float rho, float E0, uint64_t h0, int n, float* Eo,
                          float* co, int* jo, float* uxo, float* uyo, cudaStream_t st) {
     int threads = 256, blocks = (n + threads - 1) / threads;
     k_probe<<<blocks, threads, 0, st>>>(P, m, rho, E0, h0, n, Eo, co, jo, uxo, uyo);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sum_u64(const unsigned long long* v, size_t n, unsigned long long* out, int num_sms,
-                           cudaStream_t st) {
-    k_sum_u64<<<num_sms * 4, 256, 0, st>>>(v, n, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_convert(const unsigned long long* edep, const float* rho, size_t nv, double unit_J,
-                           double vol_kg_per_rho, double* dose, int num_sms, cudaStream_t st) {
-    int blocks = num_sms * 4;
-    k_convert<double><<<blocks, 256, 0, st>>>(edep, rho, nv, unit_J, vol_kg_per_rho, dose);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_convert_f32(const unsigned long long* edep, const float* rho, size_t nv, double unit_J,
-                               double vol_kg_per_rho, float* dose, int num_sms, cudaStream_t st) {
-    int blocks = num_sms * 4;
-    k_convert<float><<<blocks, 256, 0, st>>>(edep, rho, nv, unit_J, vol_kg_per_rho, dose);
     return cudaGetLastError();
 }
 
