@@ -310,7 +310,7 @@ int sde_conv3d_wgrad(const void* d_x, const void* d_dy, float* d_dw, int batch, 
 /* d_wd[ci][26 - tap][co] = d_w[co][tap][ci] (BF16): weights of the data-gradient convolution. */
 int sde_conv3d_flip_weights(const void* d_w, void* d_wd, int Cin, int Cout, void* stream);
 
-/* Host-only inspection of the work decompositions the two convolution kernels launch
+/* Host-only inspection of the work decompositions of the two convolution kernels
  * (no CUDA call: usable without a GPU, e.g. to check a shape's shared-memory and
  * tensor-memory layout before running it).
  * sde_conv3d_plan: the plan of sde_conv3d_forward for this shape, as 17 ints in the
@@ -321,16 +321,27 @@ int sde_conv3d_flip_weights(const void* d_w, void* d_wd, int Cin, int Cout, void
  * weight offset in a stage, resident weights, bytes per stage, accumulators,
  * offset of the fold's exchange buffer, tensor-memory columns, work items), and
  * its dynamic shared memory in bytes.
- * sde_conv3d_wgrad_plan: the plan of sde_conv3d_wgrad on a GPU with `sms`
+ * sde_conv3d_wgrad_plan: the row-block plan of sde_conv3d_wgrad on a GPU with `sms`
  * multiprocessors, as 14 ints: Ty, nyb, P, Yb, Nc, ntap, ngroups, kst, plane_dy,
  * plane_x, x_off, stage, items, G (input channels and taps per pass, tap groups,
  * 16-position K steps per item, plane pitches of the output-gradient rows and of
  * the input brick, brick offset in a stage, CTAs per pass), and its dynamic shared
- * memory.  Both fill min(n_fields, count) ints; SDE_EINVAL for a shape the
- * convolution rejects or has no plan for. */
+ * memory.  The weight gradient accepts the shapes that have such a plan.
+ * sde_conv3d_wgrad_ring: what it launches for them, as 19 ints: order, Ty, gpp, ngr, ns,
+ * nt, kst, P, ra, drun, dyx, xoff, dslot, xslot, DS, XS, x_off, items, G (order of the
+ * items: 0 contiguous rows, 1 the row-block plan's; rows per item, 8-channel groups
+ * per pass, row groups in N, shifted copies of the output-gradient rows in M, offsets
+ * of the x window, 16-position K steps per item, W + 2, bytes of an 8-channel run and
+ * of what is copied into it, x of its first position, the x window's first
+ * position, bytes of an output-gradient slot and of a plane slot, slots of each,
+ * offset of the first plane slot, items, CTAs per pass), and its dynamic shared memory.
+ * All fill min(n_fields, count) ints; SDE_EINVAL for a shape the convolution rejects or
+ * has no plan for. */
 int sde_conv3d_plan(int batch, int D, int H, int W, int Cin, int Cout, int32_t* fields, int n_fields,
                     uint64_t* smem_bytes);
 int sde_conv3d_wgrad_plan(int batch, int D, int H, int W, int Cin, int Cout, int sms, int32_t* fields,
+                          int n_fields, uint64_t* smem_bytes);
+int sde_conv3d_wgrad_ring(int batch, int D, int H, int W, int Cin, int Cout, int sms, int32_t* fields,
                           int n_fields, uint64_t* smem_bytes);
 
 /* Wait for the stream and report (and clear) a timed-out tensor-core wait of any

@@ -34,7 +34,7 @@ EXPORTED = [
     "sde_conv3d_flip_weights", "sde_denoise_status", "sde_denoiser_create", "sde_denoiser_destroy",
     "sde_denoiser_set_stream", "sde_denoiser_num_params", "sde_denoiser_infer", "sde_denoiser_train_step",
     "sde_denoiser_gradients", "sde_denoiser_get_params", "sde_denoiser_set_params", "sde_gamma3d",
-    "sde_scale_f32", "sde_conv3d_plan", "sde_conv3d_wgrad_plan",
+    "sde_scale_f32", "sde_conv3d_plan", "sde_conv3d_wgrad_plan", "sde_conv3d_wgrad_ring",
 ]
 
 
@@ -158,6 +158,7 @@ def lib():
         L.sde_conv3d_flip_weights.argtypes = [vp, vp, i, i, vp]
         L.sde_conv3d_plan.argtypes = [i, i, i, i, i, i, C.POINTER(C.c_int32), i, C.POINTER(u64)]
         L.sde_conv3d_wgrad_plan.argtypes = [i, i, i, i, i, i, i, C.POINTER(C.c_int32), i, C.POINTER(u64)]
+        L.sde_conv3d_wgrad_ring.argtypes = [i, i, i, i, i, i, i, C.POINTER(C.c_int32), i, C.POINTER(u64)]
         L.sde_denoise_status.argtypes = [vp]
         L.sde_denoiser_create.argtypes = [C.POINTER(vp), i, i, i, i, u64]
         L.sde_denoiser_destroy.argtypes = [vp]
@@ -434,6 +435,8 @@ CONV_PLAN_FIELDS = ("Ty", "tiles", "rowtile", "fold", "nyb", "P", "Yb", "Cp", "n
                     "stage", "nacc", "xch", "tcols", "items")
 WGRAD_PLAN_FIELDS = ("Ty", "nyb", "P", "Yb", "Nc", "ntap", "ngroups", "kst", "plane_dy", "plane_x", "x_off", "stage",
                      "items", "G")
+WGRAD_RING_FIELDS = ("order", "Ty", "gpp", "ngr", "ns", "nt", "kst", "P", "ra", "drun", "dyx", "xoff", "dslot", "xslot",
+                     "DS", "XS", "x_off", "items", "G")
 
 
 def conv3d_plan(batch, D, H, W, Cin, Cout):
@@ -446,12 +449,21 @@ def conv3d_plan(batch, D, H, W, Cin, Cout):
 
 
 def conv3d_wgrad_plan(batch, D, H, W, Cin, Cout, sms=152):
-    """Work decomposition sde_conv3d_wgrad launches on a GPU with ``sms`` multiprocessors
-    (host only, no GPU): a dict of the plan's fields plus ``smem``."""
+    """Row-block plan of sde_conv3d_wgrad on a GPU with ``sms`` multiprocessors, which the
+    accepted shapes have (host only, no GPU): a dict of the plan's fields plus ``smem``."""
     f = (C.c_int32 * len(WGRAD_PLAN_FIELDS))()
     sm = C.c_uint64()
     _check(lib().sde_conv3d_wgrad_plan(batch, D, H, W, Cin, Cout, sms, f, len(f), C.byref(sm)))
     return dict(zip(WGRAD_PLAN_FIELDS, list(f)), smem=sm.value)
+
+
+def conv3d_wgrad_ring(batch, D, H, W, Cin, Cout, sms=152):
+    """What sde_conv3d_wgrad launches on a GPU with ``sms`` multiprocessors (host only, no
+    GPU): a dict of its rings' fields plus ``smem``."""
+    f = (C.c_int32 * len(WGRAD_RING_FIELDS))()
+    sm = C.c_uint64()
+    _check(lib().sde_conv3d_wgrad_ring(batch, D, H, W, Cin, Cout, sms, f, len(f), C.byref(sm)))
+    return dict(zip(WGRAD_RING_FIELDS, list(f)), smem=sm.value)
 
 
 def conv3d_wgrad(x, dy, dw, stream=None):

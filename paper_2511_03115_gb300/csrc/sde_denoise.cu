@@ -639,177 +639,300 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 }
 
 // ----------------------------------------------------------------------------
-// Brick weight gradient: dW[co][tap][ci] = sum over output positions v of
-// dy[v][co] x[v + off(tap)][ci].  Per work item (Ty output rows of one z plane) the
-// output-gradient rows and the zero-padded input brick are staged once, both as 8-channel
-// planes with 16 bytes per position, i.e. M/N-major core matrices (8 positions x 8
-// channels); both tensors are padded channel-group-major, so each 8-channel plane of the
-// rows, and each (8-channel plane, z plane) part of the brick, is one bulk copy.  The MMA's A operand is dy (M = co, padded to 128: rows past Cout read
-// whatever follows and are never stored), K = 16 positions; B is the brick read from the
-// tap's offset (N = Nc input channels).  All taps of the pass use the same A, so the
-// tensor core fetches it once per K step.  dW accumulates in tensor memory over all the
-// CTA's items and is added to global memory once, at the end.  Padding positions of dy
-// are zero, so brick positions under them contribute nothing -- provided they hold no
-// NaN or Inf: the few positions B reads just outside the staged data (before the first
-// plane, between planes, after the last) are zeroed once at start and never written.
+// Weight gradient: dW[co][tap][ci] = sum over output voxels v of dy[v][co] x[v + off(tap)][ci].
+//
+// One MMA has K = 16 consecutive positions of an item (Ty rows of one z plane), both operands
+// M/N-major core matrices (8 positions x 8 channels), and takes as many of the 27 taps as fit it:
+//  - N is the x rows y-1 .. y+1 of the planes z-1 .. z+1 for gpp groups of eight input channels: a
+//    plane's slot in shared memory is [gpp][Ty+2][W+2] positions of 16 bytes, exactly the contiguous
+//    rows of the padded tensor, and the slots follow each other, so rows, groups and planes all
+//    lie at one stride (for Ty = 1 and gpp = 2 nine rows of 16 channels, N = 144);
+//  - dx comes from nt offsets t at which the window of x is read, each an accumulator of its own,
+//    and from ns copies of the dy row in M, shifted by s positions: dx = s + t.
+//
+// Two orders of the items, as FP32 accumulation has to go (its error grows with the number of
+// positions in a sum; 5e-5 of the gradient at 32 channels of a 192x128x128 volume, more than
+// results may move by):
+//  - short sums: a CTA owns a contiguous range of rows (Ty = 1) with z running fastest, so each
+//    further row needs one new plane; M is filled with shifted copies (ns = 3 up to 40 channels,
+//    2 up to 64), i.e. 96 of its 128 rows at 32 channels.  Positions past W up to the K step's end
+//    meet zeros in dy (its slots are zeroed once and only W positions are ever written);
+//  - long sums: the items, K steps and CTAs of the row-block plan in their order, so that every
+//    sum is formed from the same products in the same order as with one MMA per tap (bit for bit
+//    up to the order of the CTAs' atomics); three offsets t, no copies.
+//
+// One thread in each of warps 0-7 brings operands, its share of an item's 10 to 20 bulk copies; one
+// in each of warps 8-10 issues the MMAs of one offset t.  Each of these threads runs alone in its
+// warp at some seven cycles an instruction, so they keep positions, slots and phases by
+// increments: with the index divisions in their loops (three to four thousand cycles an item)
+// they, not the MMAs, set the time.  An item's commits release its dy slot and the planes no later
+// item needs.  dW stays in tensor memory over all of the CTA's items and is added to global memory
+// at the end, each CTA starting at another column (all walking the same order would meet on the
+// same addresses).
+//
+// Bound by the MMAs (N / 2 cycles each: the dense rate, a quarter of M used by 32 channels of the
+// long sums, three quarters of the short ones).  Before, one MMA a tap with 16 or 32 channels in N
+// and the x brick loaded once per tap group: 32 -> 32 channels on 192x128x128 0.915 -> 0.435 ms (long
+// order, 87 % of the MMAs' time), 64 -> 96 on 66x54x128 0.316 -> 0.149 ms (short order).
 // ----------------------------------------------------------------------------
-// The weight-gradient MMAs of one K step for taps T0 .. T1-1 (fully unrolled) of a pass
-// whose first tap is P0: the accumulator of tap t starts at column (t - P0) Nc, B's start
-// field is the K step's plus the tap's brick offset.
-template <int P0, int T0, int T1>
-__device__ __forceinline__ void wgrad_taps(uint32_t tbase, int Nc, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                           uint32_t b_hi, uint32_t idesc, uint32_t accum, const int (&toff)[27]) {
+constexpr int kRingMaxX = 12, kRingMaxD = 4, kRingCopyWarps = 8, kRingWarps = kRingCopyWarps + 3;
+
+// The MMAs of one item, offset and run of planes.  Unrolled, because address arithmetic between
+// two MMAs of one thread costs more than the MMA.
+__device__ __forceinline__ void ring_mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, int kst, uint32_t first) {
+    const uint32_t a_hi = (uint32_t)(ad >> 32), b_hi = (uint32_t)(bd >> 32);
+    uint32_t a_lo = (uint32_t)ad, b_lo = (uint32_t)bd;
+    umma::mma_bf16_lohi(d, a_lo, a_hi, b_lo, b_hi, idesc, first);
+    int ks = 1;
+    for (; ks + 4 <= kst; ks += 4) {
 #pragma unroll
-    for (int t = T0; t < T1; ++t)
-        umma::mma_bf16_lohi(tbase + (uint32_t)((t - P0) * Nc), a_lo, a_hi, b_lo + (uint32_t)toff[t], b_hi, idesc,
-                            accum);
+        for (int u = 1; u <= 4; ++u) umma::mma_bf16_lohi(d, a_lo + 16 * u, a_hi, b_lo + 16 * u, b_hi, idesc, 1u);
+        a_lo += 64;
+        b_lo += 64;
+    }
+    for (; ks < kst; ++ks) {
+        a_lo += 16;
+        b_lo += 16;
+        umma::mma_bf16_lohi(d, a_lo, a_hi, b_lo, b_hi, idesc, 1u);
+    }
 }
 
-__global__ void __launch_bounds__(192, 1) k_wgrad_brick(WgradArgs a, WgradPlan b) {
+// A CTA's items in their order: z plane, row block and sample, by increments.
+struct RingItems {
+    int left;           // items still to come, this one included
+    int z, yb, n;       // z plane, row block, sample
+    int sz, syb;        // step in (row block, z plane)
+    __device__ __forceinline__ RingItems(const WgradRing& b, int D) {
+        const long long G = gridDim.x;
+        int item;
+        if (b.order) {
+            item = blockIdx.x;
+            left = (b.items - item + (int)G - 1) / (int)G;
+            sz = (int)G % D;
+            syb = (int)G / D;
+        } else {
+            item = (int)(b.items * (long long)blockIdx.x / G);
+            left = (int)(b.items * (blockIdx.x + 1ll) / G) - item;
+            sz = 1;
+            syb = 0;
+        }
+        z = item % D;
+        yb = item / D % b.nyb;
+        n = item / D / b.nyb;
+    }
+    // Whether the next item shares two planes with this one.
+    __device__ __forceinline__ bool shares(const WgradRing& b, int D) const { return !b.order && z + 1 < D && left > 1; }
+    __device__ __forceinline__ void next(const WgradRing& b, int D) {
+        --left;
+        z += sz;
+        yb += syb;
+        if (z >= D) {
+            z -= D;
+            ++yb;
+        }
+        for (; yb >= b.nyb; yb -= b.nyb) ++n;
+    }
+};
+
+// A slot of a ring and the parity of how often the ring was gone round.
+struct RingSlot {
+    int i = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void advance(int n) {
+        if (++i == n) {
+            i = 0;
+            par ^= 1u;
+        }
+    }
+};
+
+__global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, WgradRing b) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int Cin = a.Cin, Cout = a.Cout, W = a.W, H = a.H, D = a.D, Nc = b.Nc;
-    const int P = b.P, Yb = b.Yb;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem);  // [kPipeStages]
-    uint64_t* empty = full + kPipeStages;                 // [kPipeStages]
-    uint64_t* dfull = empty + kPipeStages;                // all MMAs of the CTA done
-    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 128);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 132);
-    const uint32_t s_stage0 = umma::smem_addr(smem) + kPipeHeader;
-    const int pass = blockIdx.y;
-    const int c = pass / b.ngroups;  // input-channel chunk
-    const int t0 = (pass % b.ngroups) * b.ntap;
-    const int t1 = t0 + b.ntap < 27 ? t0 + b.ntap : 27;
-    const int my_items =
-        b.items > (int)blockIdx.x ? (b.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    {  // zero both stages: gaps around the staged data must read as 0, not leftover bits
+    const int Cin = a.Cin, Cout = a.Cout, W = a.W, H = a.H, D = a.D, Yb = b.Ty + 2;
+    uint64_t* fullx = reinterpret_cast<uint64_t*>(smem);  // [XS] plane landed
+    uint64_t* emptyx = fullx + kRingMaxX;                  // [XS] no later MMA reads the plane
+    uint64_t* fulld = emptyx + kRingMaxX;                  // [DS] dy rows landed
+    uint64_t* emptyd = fulld + kRingMaxD;                  // [DS] item's MMAs finished
+    uint64_t* dfull = emptyd + kRingMaxD;                  // all MMAs of the CTA finished
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 320);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 324);
+    const uint32_t s_d = umma::smem_addr(smem) + kPipeHeader, s_x = umma::smem_addr(smem) + (uint32_t)b.x_off;
+    const int c = blockIdx.y;  // chunk of 8 gpp input channels
+    {  // what the copies never write must read as zero, not leftover bits (0 x NaN is NaN)
         uint4* z = reinterpret_cast<uint4*>(smem + kPipeHeader);
-        const int n16 = kPipeStages * b.stage / 16;
-        for (int i = tid; i < n16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
-        umma::fence_async_smem();  // generic-proxy stores -> tensor-core reads
+        for (int i = tid; i < (b.smem - kPipeHeader) / 16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
+        umma::fence_async_smem();  // generic-proxy stores -> copies and tensor-core reads
     }
     if (warp == 0) {
         umma::tmem_alloc(slot, 512u);
         umma::tmem_relinquish();
     }
     if (tid == 0) {
-        for (int s = 0; s < kPipeStages; ++s) {
-            umma::mbar_init(&full[s], 1);
-            umma::mbar_init(&empty[s], 2);  // one commit per MMA thread
+        for (int i = 0; i < b.XS; ++i) {
+            umma::mbar_init(&fullx[i], 1);
+            umma::mbar_init(&emptyx[i], b.nt);  // one commit per issuer
         }
-        umma::mbar_init(dfull, 2);
+        for (int i = 0; i < b.DS; ++i) {
+            umma::mbar_init(&fulld[i], 1);
+            umma::mbar_init(&emptyd[i], b.nt);
+        }
+        umma::mbar_init(dfull, b.nt);
         *abort_flag = 0;
     }
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tbase = *slot;
-    const int fB = (Yb + 1) * P;  // brick position under output position 0 of the item
+    const int N = 8 * b.ngr;  // columns of an accumulator
+    RingItems it(b, D);
+    const bool any = it.left > 0;
 
-    if (warp >= 4) {
-        // two MMA threads split each pass's taps (each tap has its own accumulator columns)
-        const int iss = warp - 4;
+    if (warp < kRingCopyWarps) {
         if (lane == 0) {
-            const uint32_t idesc = umma::idesc_bf16_f32(128, Nc, 1, 1);
-            int toff[27];  // tap (dz, dy, dx) -> brick position offset (dz Yb + dy) P + dx
-#pragma unroll
-            for (int t = 0; t < 27; ++t) toff[t] = ((t / 9 - 1) * Yb + ((t / 3) % 3 - 1)) * P + (t % 3 - 1);
+            const Pcg pg{D, H, W};
+            const int gd = Cout >> 3, nd = b.ns * gd, gx = Cin >> 3;
+            const uint32_t xrun = (uint32_t)(Yb * b.P * 16);
+            const size_t plane = (size_t)(H + 2) * b.P * 16, vp = pg.vp() * 16;
+            // this warp's dy copies (copy i / gd of channel group i % gd; at most 16 in all) and the
+            // plane copies' sources, at z = y0 = n = 0
+            const unsigned char* dsrc[2];
+            uint32_t ddst[2];
+            bool mine[2];
+            for (int e = 0; e < 2; ++e) {
+                const int i = warp + kRingCopyWarps * e, s = i / gd, q = i - s * gd;
+                mine[e] = i < nd;
+                dsrc[e] = reinterpret_cast<const unsigned char*>(a.dy + 8 * pg.unit(0, gd, q, 0, 0, b.dyx - s));
+                ddst[e] = s_d + (uint32_t)(i * b.ra);
+            }
+            const unsigned char* xsrc =
+                reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.gpp, -1, -1, -1));
+            RingSlot sd, sx;
+            int j = 0, turn = nd, fresh = 3;  // fresh: planes this item brings; turn: copies go round the warps
+            size_t planes = 0;
             bool ok = true;
-            for (int j = 0; j < my_items && ok; ++j) {
-                const int s = j % kPipeStages, u = j / kPipeStages;
-                if (!pipe_wait(&full[s], (uint32_t)u & 1u, abort_flag)) {
-                    ok = false;
-                    break;
+            for (; it.left > 0; ++j) {
+                if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
+                const size_t at = (size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16);
+                if (warp == 0) umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (mine[e])
+                        umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
+                                       (uint32_t)b.drun, &fulld[sd.i]);
+                const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
+                for (int f = 0; f < fresh; ++f, ++planes) {
+                    // in the long order a plane slot goes with the dy slot that was waited for
+                    if (!b.order && planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag)))
+                        break;
+                    if (warp == 0) umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
+                    for (int q = 0; q < b.gpp; ++q, ++turn)
+                        if (turn % kRingCopyWarps == warp)
+                            umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
+                                           &fullx[sx.i]);
+                    xat += plane;
+                    sx.advance(b.XS);
                 }
+                if (!ok) break;
+                fresh = it.shares(b, D) ? 1 : 3;
+                sd.advance(b.DS);
+                it.next(b, D);
+            }
+            if (!ok) *abort_flag = 1;  // an expected copy may not come: no one may wait for it
+        }
+        __syncwarp();
+    } else if (warp - kRingCopyWarps < b.nt) {  // issuer of offset t
+        const int t = warp - kRingCopyWarps;
+        if (lane == 0) {
+            const uint32_t d = tbase + (uint32_t)(t * N);
+            // leading byte offset = next 8 positions (K); stride = next 8 channels of dy, next row,
+            // 8-channel group or plane of x
+            const uint64_t a0 = umma::smem_desc(s_d, 128, (uint32_t)b.ra);
+            const uint64_t b0 = umma::smem_desc((uint32_t)((int)s_x + 16 * (b.xoff + t)), 128, (uint32_t)b.P * 16u);
+            const uint32_t idesc = umma::idesc_bf16_f32(128, N, 1, 1);
+            const int gp = b.gpp * Yb;  // row groups of a plane
+            RingSlot sd, seen;
+            int k = 0, fresh = 3;  // k: slot of the z-1 plane
+            uint32_t accum = 0;
+            bool ok = true;
+            while (it.left > 0) {
+                for (int f = 0; ok && f < fresh; ++f) {
+                    ok = pipe_wait(&fullx[seen.i], seen.par, abort_flag);
+                    seen.advance(b.XS);
+                }
+                ok = ok && pipe_wait(&fulld[sd.i], sd.par, abort_flag);
+                if (!ok) break;
                 umma::fence_after_sync();
-                const uint32_t st = s_stage0 + (uint32_t)(s * b.stage);
-                // M/N-major: leading byte offset = next 8 positions (K), stride = next 8 channels
-                const uint64_t a0 = umma::smem_desc(st, 128, (uint32_t)b.plane_dy);
-                const uint64_t b0 = umma::smem_desc(st + (uint32_t)b.x_off, 128, (uint32_t)b.plane_x);
-                const uint32_t a_hi = (uint32_t)(a0 >> 32), b_hi = (uint32_t)(b0 >> 32);
-                for (int ks = 0; ks < b.kst; ++ks) {
-                    const uint32_t a_lo = (uint32_t)a0 + (uint32_t)(16 * ks);  // 16 positions of 16 bytes
-                    const uint32_t b_lo = (uint32_t)b0 + (uint32_t)(fB + 16 * ks);
-                    // each tap's accumulator starts at its first MMA: item 0, K step 0
-                    const uint32_t accum = (j > 0 || ks > 0) ? 1u : 0u;
-                        // unrolled over this pass's taps: one add per instruction; fB + offset >= -1,
-                    // one position before the brick at most (dy is zero there), so the start
-                    // field never borrows
-                    if (t0 == 0 && t1 == 27) {
-                        if (iss) wgrad_taps<0, 14, 27>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                        else wgrad_taps<0, 0, 14>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                    } else if (t0 == 0 && t1 == 14) {
-                        if (iss) wgrad_taps<0, 7, 14>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                        else wgrad_taps<0, 0, 7>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                    } else if (t0 == 14 && t1 == 27) {
-                        if (iss) wgrad_taps<14, 21, 27>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                        else wgrad_taps<14, 14, 21>(tbase, Nc, a_lo, a_hi, b_lo, b_hi, idesc, accum, toff);
-                    } else
-                        for (int t = t0 + iss; t < t1; t += 2)
-                            umma::mma_bf16_lohi(tbase + (uint32_t)((t - t0) * Nc), a_lo, a_hi,
-                                                b_lo + (uint32_t)(((t / 9 - 1) * Yb + ((t / 3) % 3 - 1)) * P +
-                                                                  (t % 3 - 1)),
-                                                b_hi, idesc, accum);
+                // descriptors step by their start field, in 16-byte units
+                const uint64_t ad = a0 + (uint32_t)(sd.i * (b.dslot >> 4)), bd = b0 + (uint32_t)(k * (b.xslot >> 4));
+                const int run = b.XS - k;  // planes before the ring wraps
+                if (run >= 3) {
+                    ring_mma(d, ad, bd, idesc, b.kst, accum);
+                } else {
+                    const int n1 = run * gp;
+                    ring_mma(d, ad, bd, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, accum);
+                    ring_mma(d + (uint32_t)(8 * n1), ad, b0, umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, accum);
                 }
-                umma::mma_commit(&empty[s]);
+                accum = 1;
+                umma::mma_commit(&emptyd[sd.i]);
+                sd.advance(b.DS);
+                fresh = it.shares(b, D) ? 1 : 3;
+                if (b.order) {
+                    k = k + 3 < b.XS ? k + 3 : 0;
+                } else {
+                    for (int f = 0; f < fresh; ++f) {
+                        umma::mma_commit(&emptyx[k]);
+                        k = k + 1 < b.XS ? k + 1 : 0;
+                    }
+                }
+                it.next(b, D);
             }
             if (ok) umma::mma_commit(dfull);
         }
         __syncwarp();
-    } else {
-        bool ok = true;
-        auto worker_wait = [&](uint64_t* m, uint32_t parity) {
-            bool done = true;
-            if (tid == 0) done = pipe_wait(m, parity, abort_flag);
-            return workers_all<128>(done);
-        };
-        if (tid == 0) {  // producer: per item Cout/8 runs of dy rows and Nc/8 x 3 runs of the input brick
-            const Pcg pg{D, H, W};
-            const uint32_t run_dy = (uint32_t)(b.Ty * P * 16), run_x = (uint32_t)(Yb * P * 16);
-            const int gdy = Cout >> 3, gx = Nc >> 3;
-            int j = 0;
-            for (; j < my_items; ++j) {
-                const int s = j % kPipeStages, u = j / kPipeStages;
-                if (u >= 1 && !pipe_wait(&empty[s], (uint32_t)(u - 1) & 1u, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                int r = (int)blockIdx.x + j * (int)gridDim.x;
-                const int z = r % D;
-                r /= D;
-                const int y0 = (r % b.nyb) * b.Ty;
-                const int n = r / b.nyb;
-                const uint32_t st = s_stage0 + (uint32_t)(s * b.stage);
-                umma::mbar_arrive_expect_tx(&full[s], (uint32_t)gdy * run_dy + (uint32_t)(3 * gx) * run_x);
-                // output-gradient rows y0 .. y0+Ty-1 with their zero padding columns; the
-                // positions up to kst*16 past them stay zero from the start
-                for (int q = 0; q < gdy; ++q)
-                    umma::bulk_g2s(st + (uint32_t)(q * b.plane_dy), a.dy + 8 * pg.unit(n, gdy, q, z, y0, -1), run_dy,
-                                   &full[s]);
-                for (int g = 0; g < gx; ++g)
-                    for (int zb = 0; zb < 3; ++zb)
-                        umma::bulk_g2s(st + (uint32_t)(b.x_off + g * b.plane_x) + (uint32_t)zb * run_x,
-                                       a.x + 8 * pg.unit(n, Cin >> 3, c * gx + g, z + zb - 1, y0 - 1, -1), run_x,
-                                       &full[s]);
-            }
-            // no copy may still be writing shared memory when the CTA exits
-            for (int jj = j > kPipeStages ? j - kPipeStages : 0; jj < j; ++jj)
-                umma::mbar_wait(&full[jj % kPipeStages], (uint32_t)(jj / kPipeStages) & 1u, kWaitCycles);
+    }
+    __syncthreads();
+    if (*abort_flag) {
+        // copies of some item may still be in flight: every barrier's current phase ends when
+        // its own copies have landed, or was never armed; wait for the ones that were
+        if (tid == 0) {
+            for (int i = 0; i < b.DS; ++i)
+                for (int ph = 0; ph < 2; ++ph) umma::mbar_wait(&fulld[i], (uint32_t)ph, kWaitCycles >> 6);
+            for (int i = 0; i < b.XS; ++i)
+                for (int ph = 0; ph < 2; ++ph) umma::mbar_wait(&fullx[i], (uint32_t)ph, kWaitCycles >> 6);
         }
-        ok = workers_all<128>(ok);
-        if (ok && my_items > 0 && worker_wait(dfull, 0u)) {
+    } else if (warp < 8) {
+        bool ok = true;
+        if (tid == 0) ok = pipe_wait(dfull, 0u, abort_flag);
+        ok = workers_all<256>(ok);
+        if (ok && any) {
             umma::fence_after_sync();
-            const int co = 32 * warp + lane;
-            if (32 * warp < Cout) {  // warp-uniform: lanes past Cout load but do not store
-                for (int t = t0; t < t1; ++t)
-                    for (int cc = 0; cc < Nc; cc += 8) {
-                        float v[8];
-                        __syncwarp();
-                        umma::tmem_ld8(tbase + ((uint32_t)(32 * warp) << 16) + (uint32_t)((t - t0) * Nc + cc), v);
-                        if (co < Cout)
-                            for (int e = 0; e < 8; ++e)
-                                atomicAdd(&a.dw[((size_t)co * 27 + t) * Cin + c * Nc + cc + e], v[e]);
+            const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. + 31; two warps share them
+            const int m = 32 * quarter + lane, i = m / Cout, co = m - i * Cout;  // row: copy i of channel co
+            const bool vec = (reinterpret_cast<uintptr_t>(a.dw) & 15) == 0;
+            const int cells = b.nt * b.ngr;  // (offset, row group) cells of eight columns
+            if (32 * quarter < b.ns * Cout) {  // warp-uniform: lanes past the last copy load but do not store
+                int cell = (int)((blockIdx.x * 7u) % (unsigned)cells);
+                for (int n = 0; n < cells; ++n, cell = cell + 1 < cells ? cell + 1 : 0) {
+                    if ((n & 1) != (warp >> 2)) continue;
+                    const int t = cell / b.ngr, q = cell - t * b.ngr;
+                    const int r = q % Yb, pg = q / Yb, dz = pg / b.gpp, g = pg - dz * b.gpp;
+                    const int dx = t + i - 1;
+                    if (r > 2 || dz > 2) continue;  // rows between the taps
+                    float v[8];
+                    __syncwarp();
+                    umma::tmem_ld8(tbase + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(t * N + 8 * q), v);
+                    // two copies give dx = 0 twice, the second time (s = 1, t = -1) without the last position
+                    if (i < b.ns && !(b.ns == 2 && i == 1 && t == 0)) {
+                        float* d = a.dw + ((size_t)co * 27 + 9 * dz + 3 * r + dx + 1) * Cin + 8 * (c * b.gpp + g);
+                        if (vec) {
+                            atomicAdd(reinterpret_cast<float4*>(d), make_float4(v[0], v[1], v[2], v[3]));
+                            atomicAdd(reinterpret_cast<float4*>(d) + 1, make_float4(v[4], v[5], v[6], v[7]));
+                        } else {
+                            for (int e = 0; e < 8; ++e) atomicAdd(d + e, v[e]);
+                        }
                     }
+                }
             }
         }
     }
@@ -967,11 +1090,10 @@ cudaError_t conv3d_launch(const ConvArgs& a, int batch, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Plan of the brick weight gradient: Nc in {16, 32} input channels per pass, as many
-// taps per pass as 512 tensor-memory columns hold, and Ty a divisor of H whose two stages
-// fit; the cost model (~56 cycles per MMA; bulk copies ~64 bytes per cycle per SM) picks
-// among them.  Measured alternative, slower on the denoiser's
-// layers: one input plane per pass with the nine taps of one dz (more rows per item).
+// Row-block plan of the weight gradient (sde_conv3d_wgrad_plan): Nc in {16, 32} input channels
+// per pass, as many taps per pass as 512 tensor-memory columns hold, and Ty a divisor of H whose
+// two stages fit.  It was the launched decomposition before the rings below; the shapes that the
+// call accepts are still those that it has a plan for.
 static bool wgrad_plan(const WgradArgs& a, int sms, WgradPlan* out, size_t* smem_out) {
     const int P = a.W + 2;
     double best = 1e300;
@@ -1015,18 +1137,80 @@ static bool wgrad_plan(const WgradArgs& a, int sms, WgradPlan* out, size_t* smem
     return found;
 }
 
+// Rings of the weight gradient for one layer shape: the order of the items by the length of its
+// sums (in K steps of the row-block plan), then as many dy slots (up to four) and plane slots (up
+// to twelve; the fewer, the more often a range's planes wrap) as fit.  At 1024 steps the short
+// order moves the gradient by about 1.2e-5 and takes half the time of the long one.
+constexpr double kLongSum = 1024.0;
+
+bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing* out) {
+    const double steps = (double)wp.items / wp.G * wp.kst;
+    // the last choice, eight channels a pass in the short order, is for rows so wide that two groups
+    // of input rows do not fit beside two dy slots of 128 channels
+    for (int choice = steps > kLongSum && wp.Ty <= 6 ? 0 : 1; choice < 3; ++choice) {
+        const int order = choice == 0 ? 1 : 0;
+        WgradRing w{};
+        w.order = order;
+        w.P = a.W + 2;
+        if (order) {
+            w.Ty = wp.Ty;
+            w.ns = 1;
+            w.gpp = wp.Ty == 1 ? 2 : 1;  // what three accumulators in tensor memory leave room for
+            w.kst = wp.kst;
+            w.drun = w.Ty * w.P * 16;  // rows with their padding, from x = -1
+            w.dyx = -1;
+            w.G = wp.G;
+        } else {
+            w.Ty = 1;
+            w.ns = a.Cout <= 40 ? 3 : a.Cout <= 64 ? 2 : 1;
+            w.gpp = choice == 1 ? 2 : 1;
+            w.kst = (a.W + 15) / 16;
+            w.drun = a.W * 16;
+            w.dyx = w.ns == 3 ? 1 : 0;  // copy 0 is shifted by s = -1 or 0
+        }
+        w.nt = w.ns == 3 ? 1 : w.ns == 2 ? 2 : 3;
+        // the window of t = t0 at the first position: the slot's rows start at x = -1
+        w.xoff = order ? -1 : w.nt == 1 ? 1 : 0;
+        w.nyb = a.H / w.Ty;
+        w.items = a.batch * w.nyb * a.D;
+        const int Yb = w.Ty + 2, passes = a.Cin / (8 * w.gpp);
+        w.ngr = ((3 * w.gpp - 1) * Yb + 3 + 1) / 2 * 2;  // N is a multiple of 16
+        w.ra = w.kst * 256;
+        w.dslot = w.ns * (a.Cout / 8) * w.ra;
+        w.xslot = w.gpp * Yb * w.P * 16;
+        if (!order) {
+            w.G = sms / passes > 1 ? sms / passes : 1;  // all passes in one wave on the SMs
+            if (w.G > w.items) w.G = w.items;
+        }
+        for (w.DS = kRingMaxD; w.DS >= 2; --w.DS)
+            for (w.XS = order ? 3 * w.DS : kRingMaxX; w.XS >= (order ? 3 * w.DS : w.DS + 2); --w.XS) {
+                w.x_off = kPipeHeader + w.DS * w.dslot;
+                // the windows of the last slot end up to a row and a K step past it, and M = 128 rows of
+                // A start in the last dy slot
+                const int tail = kPipeHeader + (w.DS - 1) * w.dslot + 16 * w.ra;
+                w.smem = w.x_off + w.XS * w.xslot + (w.P + 32) * 16;
+                if (w.smem < tail) w.smem = tail;
+                if (w.smem <= 227 * 1024) {
+                    *out = w;
+                    return true;
+                }
+            }
+    }
+    return false;
+}
+
 cudaError_t wgrad_launch(const WgradArgs& a, cudaStream_t st) {
     WgradPlan wp{};
+    WgradRing wr{};
     size_t wsmem = 0;
     int dev = 0, sms = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e0 != cudaSuccess) return e0;
-    if (!wgrad_plan(a, sms, &wp, &wsmem)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_wgrad_brick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)wp.G, (unsigned)((a.Cin / wp.Nc) * wp.ngroups));
-    k_wgrad_brick<<<grid, 192, wsmem, st>>>(a, wp);
+    if (!wgrad_plan(a, sms, &wp, &wsmem) || !wgrad_ring_plan(a, sms, wp, &wr)) return cudaErrorInvalidValue;
+    e = cudaFuncSetAttribute(k_wgrad_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, wr.smem);
+    if (e != cudaSuccess) return e;
+    k_wgrad_ring<<<dim3((unsigned)wr.G, (unsigned)(a.Cin / (8 * wr.gpp))), 32 * kRingWarps, wr.smem, st>>>(a, wr);
     return cudaGetLastError();
 }
 
@@ -1163,5 +1347,30 @@ extern "C" int sde_conv3d_wgrad_plan(int batch, int D, int H, int W, int Cin, in
                            wp.kst,      wp.plane_dy, wp.plane_x, wp.x_off, wp.stage, wp.items, wp.G};
     for (int i = 0; i < n_fields && i < 14; ++i) fields[i] = v[i];
     if (smem_bytes) *smem_bytes = smem;
+    return SDE_OK;
+}
+
+extern "C" int sde_conv3d_wgrad_ring(int batch, int D, int H, int W, int Cin, int Cout, int sms, int32_t* fields,
+                                     int n_fields, uint64_t* smem_bytes) {
+    WgradArgs a{};
+    a.D = D;
+    a.H = H;
+    a.W = W;
+    a.Cin = Cin;
+    a.Cout = Cout;
+    a.nvox = D * H * W;
+    a.batch = batch;
+    WgradRing w{};
+    WgradPlan wp{};
+    size_t smem = 0;
+    if (!conv_shape_ok(D, H, W, Cin, Cout, batch) || Cout > 128 || sms < 1 || n_fields < 0 ||
+        (n_fields > 0 && !fields) || !wgrad_plan(a, sms, &wp, &smem) || !wgrad_ring_plan(a, sms, wp, &w)) {
+        set_last_error("sde_conv3d_wgrad_ring: shape rejected by the weight gradient or without a plan");
+        return SDE_EINVAL;
+    }
+    const int32_t v[19] = {w.order, w.Ty, w.gpp, w.ngr, w.ns,  w.nt,  w.kst,  w.P,     w.ra, w.drun,
+                           w.dyx,   w.xoff, w.dslot, w.xslot, w.DS, w.XS, w.x_off, w.items, w.G};
+    for (int i = 0; i < n_fields && i < 19; ++i) fields[i] = v[i];
+    if (smem_bytes) *smem_bytes = (uint64_t)w.smem;
     return SDE_OK;
 }

@@ -94,6 +94,27 @@ struct WgradPlan {
     int G;               // CTAs per pass
 };
 
+// Order, rings and operand shapes of the weight-gradient kernel (host-chosen per layer shape).
+struct WgradRing {
+    int order;         // 0: contiguous rows per CTA (short sums), 1: the row-block plan's items (long sums)
+    int Ty, nyb;       // rows per item, H / Ty
+    int gpp;           // groups of eight input channels per pass
+    int ngr;           // row groups of N (N = 8 ngr)
+    int ns;            // copies of the dy row in M, shifted by s = -1..1 (3), 0..1 (2) or 0 (1)
+    int nt;            // offsets at which the x window is read: 0 (1), -1..0 (2) or -1..1 (3)
+    int kst;           // K steps of 16 positions per item
+    int P;             // W + 2: positions of an x row
+    int ra;            // bytes of an 8-channel run of dy (kst x 16 positions)
+    int drun, dyx;     // bytes copied into it, x of its first position in copy 0
+    int xoff;          // position in a plane's first row under the item's first position, at the first offset
+    int dslot, xslot;  // bytes of a dy slot (ns x Cout/8 runs) and of a plane slot (gpp x (Ty + 2) rows)
+    int DS, XS;        // dy slots and plane slots
+    int x_off;         // offset of the first plane slot
+    int smem;          // dynamic shared memory in bytes
+    int items;         // batch x nyb x D
+    int G;             // CTAs per pass
+};
+
 // Output channels per part that conv3d_launch will use for this layer shape (the packing
 // of its weights), or 0 if the shape has no plan.
 int conv_plan_cp(int D, int H, int W, int Cin, int Cout);
