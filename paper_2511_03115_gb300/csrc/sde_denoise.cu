@@ -200,22 +200,32 @@ namespace {
 // otherwise M tiles of 128 consecutive positions cover the Ty rows including their
 // padding columns and the epilogue drops the rows that are not output voxels.
 //
-// Persistent and warp-specialised: the producer warp streams (brick, weight) chunks into
-// a ring of shared-memory stages, one bulk copy per lane (each stage's "full" barrier
-// completes when the bytes of its copies have landed); one thread in each of two MMA
-// warps issues tcgen05.mma for the M tiles of its parity into one of two tensor-memory
-// accumulators, and both release stages and accumulators through tcgen05.commit; the
-// kConvWorkers epilogue warps turn a finished accumulator into output (bias, leaky ReLU,
-// BF16 or FP32 store) while the tensor core works on the next item.  Every wait is bounded; a timeout sets a shared abort flag that
-// ends all roles' loops, and the producer waits for its copies in flight before the CTA
+// Persistent and warp-specialised: one thread in each of three copy warps, one per plane of the
+// brick, streams that plane's runs and weights into a ring of shared-memory stages (a "full"
+// barrier per stage and plane completes when the bytes of its copies have landed); two MMA
+// warps issue tcgen05.mma for the M tiles of their parity, plane by plane, into one of two
+// tensor-memory accumulators, and release planes and accumulators through tcgen05.commit; the
+// epilogue groups turn a finished tile into output (bias, leaky ReLU, BF16 or FP32 store) while the
+// tensor core works on the next ones.  Every wait is bounded; a timeout sets a shared abort flag
+// that ends all roles' loops, and each copy thread waits for its copies in flight before the CTA
 // exits.
+//
+// The copy and MMA roles run one warp each, at some seven cycles an instruction, so their loops
+// hold no index division, no dispatch and no address that a step could carry: with those a plane
+// took them 500 cycles whatever its MMAs (100 to 500).  The stages are released a plane at a time,
+// which with two of them keeps five of six planes in flight.  192x128x128: 16 -> 32 channels 150 ->
+// 117 us, 32 -> 32 200 -> 165 (the folded epilogue bounds it: 110 without), 96 -> 32 472 -> 336 (operand
+// reads and copies share the shared memory's port), inference 1.89 -> 1.55 ms.
 // ----------------------------------------------------------------------------
 constexpr int kPipeStages = 2;
 constexpr int kPipeHeader = 1024;  // barriers, tensor-memory slot, abort flag
 
+// One try first: the clock and the abort flag cost a role that runs alone in its warp more than
+// the wait when the phase is over already.
 __device__ __forceinline__ bool pipe_wait(uint64_t* m, uint32_t parity, volatile int* abort_flag) {
+    if (umma::mbar_try_wait(m, parity)) return true;
     const long long t0 = clock64();
-    while (!umma::mbar_try_wait(m, parity)) {
+    while (!umma::mbar_try_wait_long(m, parity)) {
         if (*abort_flag) return false;
         if (clock64() - t0 > kWaitCycles) {
             *abort_flag = 1;
@@ -225,11 +235,13 @@ __device__ __forceinline__ bool pipe_wait(uint64_t* m, uint32_t parity, volatile
     return true;
 }
 
-// Epilogue warps of the brick convolution; two share each tensor-memory lane quarter
-// (warp & 3).  The two MMA warps and the producer warp follow them.
-constexpr int kConvWorkers = 8;
-constexpr int kConvWorkerThreads = 32 * kConvWorkers;
-constexpr int kConvThreads = kConvWorkerThreads + 96;
+// Epilogue warps of the brick convolution, groups of four that cover a tile's 128 lanes (warp &
+// 3: the tensor-memory lane quarter); the two MMA warps and the copy warps follow them.  32 -> 32
+// channels on 192x128x128: two groups 175 us, three 165, four 167.
+constexpr int kConvGroups = 3;
+constexpr int kConvWorkers = 4 * kConvGroups;
+constexpr int kConvCopyWarps = 3;  // one per brick plane
+constexpr int kConvThreads = 32 * (kConvWorkers + 2 + kConvCopyWarps);
 
 // AND of a predicate over the NT worker threads of a kernel (its warps 0 .. NT/32 - 1),
 // named barrier 1.
@@ -252,92 +264,296 @@ __device__ __forceinline__ int tile_base(int m, bool rowtile, int P, int Yb, int
     return rowtile ? (Yb + 1) * P + 1 + (m / tpr) * P + (m % tpr) * 128 : (Yb + 1) * P + 128 * m;
 }
 
-// The 27 x TILES MMAs of one channel chunk, fully unrolled so that the issuing thread spends
-// one integer add per instruction: A's start field is the stage's plus (tile base + tap
-// offset), B's steps by one tap tile (Cp x 16 BF16 = 2 Cp units of 16 bytes).  The start
-// fields stay within 14 bits (shared addresses below 256 KB, lowest start one position
-// into the stage), so adding to the low word never carries or borrows into the others.
-template <int TILES, int PAR>
-__device__ __forceinline__ void conv_chunk_mma(uint32_t dacc, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                               uint32_t b_hi, uint32_t idesc, int Cp, const int (&toff)[27],
-                                               bool rowtile, int P, int Yb, int tpr, uint32_t first_accum) {
-    int tb[TILES];
-#pragma unroll
-    for (int m = PAR; m < TILES; m += 2) tb[m] = tile_base(m, rowtile, P, Yb, tpr);
-#pragma unroll
-    for (int t = 0; t < 27; ++t) {
-        const uint32_t bl = b_lo + (uint32_t)(2 * Cp * t);
-#pragma unroll
-        for (int m = PAR; m < TILES; m += 2)
-            umma::mma_bf16_lohi(dacc + (uint32_t)(m * Cp), a_lo + (uint32_t)(tb[m] + toff[t]), a_hi, bl, b_hi, idesc,
-                                t > 0 ? 1u : first_accum);
-    }
-}
+// What an MMA warp needs beside the plan: barriers, the first stage's operand descriptors (A at
+// the plane z - 1 of tap (-1, -1, -1)'s row offset 0, B at tap 0) and the resident weights'.
+struct IssueArgs {
+    uint64_t *full, *empty, *tfull, *tempty;
+    volatile int* abort_flag;
+    uint64_t a0, b0;
+    uint32_t tbase, idesc, leader;
+    int items, nchunk, Cp, tpr;
+};
 
-// Folded variant (one 128-voxel row per tile): per (z, y) tap pair q one MMA of N = 3 Cp whose
-// B is the three consecutive x-tap tiles of the pair and whose A is the pair's dx = 0
-// window; accumulator column block j then holds the window's product with the dx = j - 1
-// weights, and the epilogue adds the blocks shifted by one position.
-template <int TILES, int PAR>
-__device__ __forceinline__ void conv_chunk_mma_fold(uint32_t dacc, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                                    uint32_t b_hi, uint32_t idesc, int Cp, const int (&toff)[27],
-                                                    int P, int Yb, uint32_t first_accum) {
-    int tb[TILES];
+// The MMA warp of the M tiles of parity PAR: per item, chunk and plane dz the taps' MMAs in order,
+// straight through with an add or two per instruction.  A warp issues alone, at some seven
+// cycles an instruction, and a plane is 3 to 9 MMAs per tile: a dispatch on the tile count and
+// descriptors formed per plane took as long as the MMAs (500 cycles a plane).
+//  - unfolded: nine taps per plane, A's start field the plane's plus tile base and tap offset, B's a
+//    tap tile (Cp x 16 BF16 = 2 Cp units of 16 bytes) further each;
+//  - folded (one 128-voxel row per tile): per (z, y) tap pair one MMA of N = 3 Cp whose B is the
+//    three consecutive x-tap tiles of the pair and whose A is the pair's dx = 0 window;
+//    accumulator column block j then holds the window's product with the dx = j - 1 weights,
+//    and the epilogue adds the blocks shifted by one position.
+// The start fields stay within 14 bits (shared addresses below 256 KB, lowest start one position
+// into the stage), so adding to the low word never carries or borrows into the others.
+template <bool FOLD, int TILES, int PAR>
+__device__ __forceinline__ void conv_issue(const BrickPlan& b, const IssueArgs& g) {
+    static_assert(kPipeStages == 2, "stages alternate");
+    const uint32_t a_hi = (uint32_t)(g.a0 >> 32), b_hi = (uint32_t)(g.b0 >> 32);
+    const int P = b.P, plane = b.Yb * P, Cp = g.Cp, acc_cols = TILES * Cp * (FOLD ? 3 : 1);
+    uint32_t tb[TILES], td[TILES];
 #pragma unroll
-    for (int m = PAR; m < TILES; m += 2) tb[m] = tile_base(m, true, P, Yb, 1);
+    for (int m = PAR; m < TILES; m += 2) {
+        tb[m] = (uint32_t)g.a0 + (uint32_t)(tile_base(m, b.rowtile != 0, P, b.Yb, g.tpr) - plane - P);
+        td[m] = (uint32_t)(m * Cp * (FOLD ? 3 : 1));
+    }
+    const uint32_t stage = (uint32_t)b.stage >> 4, w_chunk = (uint32_t)(27 * 2 * Cp);
+    uint32_t soff = 0, par = 0, acc_par = 1;
+    int acc = 0;
+    bool ok = true;
+    for (int j = 0; j < g.items; ++j) {
+        if (j >= b.nacc) ok = pipe_wait(&g.tempty[acc], acc_par, g.abort_flag);
+        const uint32_t dacc = g.tbase + (uint32_t)(acc * acc_cols);
+        for (int c = 0; c < g.nchunk; ++c) {
+            uint64_t* const full = g.full + (soff ? 3 : 0);
+            uint64_t* const empty = g.empty + (soff ? 3 : 0);
+            const uint32_t bs = (uint32_t)g.b0 + (b.wres ? (uint32_t)c * w_chunk : soff);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const uint32_t bl = b_lo + (uint32_t)(6 * Cp * q);  // taps 3q .. 3q+2
+            for (int dz = 0; dz < 3; ++dz) {
+                ok = ok && pipe_wait(&full[dz], par, g.abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) return;
+                umma::fence_after_sync();
+                const uint32_t as = soff + (uint32_t)(dz * plane), bz = bs + (uint32_t)(18 * Cp * dz);
+                const uint32_t first = dz > 0 || c > 0 ? 1u : 0u;
 #pragma unroll
-        for (int m = PAR; m < TILES; m += 2)
-            umma::mma_bf16_lohi(dacc + (uint32_t)(3 * m * Cp), a_lo + (uint32_t)(tb[m] + toff[3 * q + 1]), a_hi, bl,
-                                b_hi, idesc, q > 0 ? 1u : first_accum);
+                for (int q = 0; q < (FOLD ? 3 : 9); ++q) {
+                    // folded: the middle x offset of row pair q and its three tap tiles
+                    const uint32_t ao = as + (uint32_t)((FOLD ? q : q / 3) * P + (FOLD ? 0 : q % 3 - 1));
+                    const uint32_t bo = bz + (uint32_t)((FOLD ? 6 : 2) * Cp * q);
+#pragma unroll
+                    for (int m = PAR; m < TILES; m += 2)
+                        umma::mma_bf16_warp(g.leader, dacc + td[m], tb[m] + ao, a_hi, bo, b_hi, g.idesc, q > 0 ? 1u : first);
+                }
+                umma::mma_commit_warp(g.leader, &empty[dz]);
+            }
+            par ^= soff ? 1u : 0u;
+            soff = soff ? 0u : stage;
+        }
+        umma::mma_commit_warp(g.leader, &g.tfull[acc]);
+        if (++acc == b.nacc) {
+            acc = 0;
+            acc_par ^= 1u;
+        }
     }
 }
 
 // Named barrier over the 128 threads of one group of four epilogue warps.
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
-// Work item of the brick convolution: (sample, Cout part, row block, z plane).
-struct BrickItem {
-    int n, part, y0, z;
+// Work item of the brick convolution: (sample, Cout part, row block, z plane), z fastest.  A CTA
+// takes every gridDim.x-th one and steps by increments (its roles run one thread a warp, where an
+// integer division costs a hundred cycles).
+struct BrickItems {
+    int left;             // items still to come, this one included
+    int z, yb, part, n;
+    int sz, syb;          // step in (row block, z plane)
+    __device__ __forceinline__ BrickItems(const BrickPlan& b, int D) {
+        int item = blockIdx.x;
+        const int G = gridDim.x;
+        left = (b.items - item + G - 1) / G;
+        sz = G % D;
+        syb = G / D;
+        z = item % D;
+        item /= D;
+        yb = item % b.nyb;
+        item /= b.nyb;
+        part = item % b.nsplit;
+        n = item / b.nsplit;
+    }
+    __device__ __forceinline__ void next(const BrickPlan& b, int D) {
+        --left;
+        z += sz;
+        yb += syb;
+        if (z >= D) {
+            z -= D;
+            ++yb;
+        }
+        for (; yb >= b.nyb; yb -= b.nyb)
+            if (++part == b.nsplit) {
+                part = 0;
+                ++n;
+            }
+    }
 };
-__device__ __forceinline__ BrickItem brick_item(const BrickPlan& b, int D, int item) {
-    BrickItem t;
-    t.z = item % D;
-    item /= D;
-    t.y0 = (item % b.nyb) * b.Ty;
-    item /= b.nyb;
-    t.part = item % b.nsplit;
-    t.n = item / b.nsplit;
-    return t;
+
+// Sixteen accumulator columns of this lane's row of a tile, from tcol on, as packed pairs.
+// Folded: out[x] = D[x-1][co] + D[x][Cp + co] + D[x+1][2 Cp + co]; x - 1 and x + 1 of a lane
+// quarter's edge lanes belong to the neighbouring quarter (another warp of the group), x = -1 and
+// x = 128 are padding (their D is zero).  Edge lanes publish their columns in xch
+// ([2][quarter][16]), all warps of the group meet, and the edge lanes add what their
+// neighbours published.
+template <bool FOLD>
+__device__ __forceinline__ void tile_columns(uint32_t tcol, int Cp, float* xch, bool one_buffer, int quarter, int lane,
+                                             int barrier, float2 (&out)[8]) {
+    uint32_t v[16];
+    if (FOLD) {
+        uint32_t lo[16], hi[16];
+        umma::tmem_ld16_nowait(tcol, lo);
+        umma::tmem_ld16_nowait(tcol + (uint32_t)(2 * Cp), hi);
+        umma::tmem_wait_ld16(lo);
+        umma::tmem_touch16(hi);
+        if (lane == 31 || lane == 0) {
+            uint4* dst = reinterpret_cast<uint4*>(xch + (lane == 31 ? 0 : 64) + quarter * 16);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                dst[q] = lane == 31 ? make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3])
+                                    : make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+        }
+        umma::tmem_ld16_nowait(tcol + (uint32_t)Cp, v);
+        const uint32_t ml = lane == 0 ? 0u : ~0u, mr = lane == 31 ? 0u : ~0u;
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+            float2 l, r;
+            l.x = __uint_as_float(__shfl_up_sync(0xffffffffu, lo[e], 1) & ml);
+            l.y = __uint_as_float(__shfl_up_sync(0xffffffffu, lo[e + 1], 1) & ml);
+            r.x = __uint_as_float(__shfl_down_sync(0xffffffffu, hi[e], 1) & mr);
+            r.y = __uint_as_float(__shfl_down_sync(0xffffffffu, hi[e + 1], 1) & mr);
+            out[e / 2] = __fadd2_rn(l, r);
+        }
+        group_sync(barrier);
+        const bool left = lane == 0;
+        if ((left && quarter > 0) || (lane == 31 && quarter < 3)) {
+            const float4* src = reinterpret_cast<const float4*>(xch + (left ? (quarter - 1) * 16 : 64 + (quarter + 1) * 16));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = src[q];
+                out[2 * q] = __fadd2_rn(make_float2(w.x, w.y), out[2 * q]);
+                out[2 * q + 1] = __fadd2_rn(make_float2(w.z, w.w), out[2 * q + 1]);
+            }
+        }
+        __syncwarp();
+        if (one_buffer) group_sync(barrier);  // the next columns go to the same buffer
+    } else {
+        umma::tmem_ld16_nowait(tcol, v);
+    }
+    umma::tmem_wait_ld16(v);
+#pragma unroll
+    for (int e = 0; e < 16; e += 2) {
+        const float2 d = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+        out[e / 2] = FOLD ? __fadd2_rn(d, out[e / 2]) : d;
+    }
+}
+
+// Where a tile's lane writes: the 16-byte unit of its voxel in the part's first channel group of y
+// (FP32 output: its voxel index), that of its first child on the doubled grid, and whether it
+// is an output voxel.
+struct TileVoxel {
+    size_t at, up;
+    bool valid;
+};
+
+// Bias, leaky ReLU and the stores of the sixteen channels from cbase + c on (tile_columns in r).
+__device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel& t, int cbase, int c, int lane, size_t vp,
+                                              float2 (&r)[8]) {
+    const int ch = cbase + c;
+    if (a.bias) {
+        const float4* bq = reinterpret_cast<const float4*>(a.bias + ch);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 w = __ldg(bq + q);
+            r[2 * q] = __fadd2_rn(r[2 * q], make_float2(w.x, w.y));
+            r[2 * q + 1] = __fadd2_rn(r[2 * q + 1], make_float2(w.z, w.w));
+        }
+    }
+    if (a.relu) {
+        const float2 slope = make_float2(a.slope, a.slope);
+        if (a.slope > 0.f) {  // 0 < slope < 1: the larger of x and slope x
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float2 s = __fmul2_rn(slope, r[e]);
+                r[e] = make_float2(fmaxf(r[e].x, s.x), fmaxf(r[e].y, s.y));
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float2 s = __fmul2_rn(slope, r[e]);
+                r[e].x = r[e].x > 0.f ? r[e].x : s.x;
+                r[e].y = r[e].y > 0.f ? r[e].y : s.y;
+            }
+        }
+    }
+    if (a.y_fp32) {
+        if (!t.valid) return;
+        if (a.y_keep) {  // leading channels only
+            if (ch == 0)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {  // constant indices keep r in registers
+                    if (2 * e < a.y_keep) static_cast<float*>(a.y)[t.at * a.y_keep + 2 * e] = r[e].x;
+                    if (2 * e + 1 < a.y_keep) static_cast<float*>(a.y)[t.at * a.y_keep + 2 * e + 1] = r[e].y;
+                }
+        } else {
+            float4* yo = reinterpret_cast<float4*>(static_cast<float*>(a.y) + t.at * a.y_cstride + a.y_coffset + ch);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) yo[q] = make_float4(r[2 * q].x, r[2 * q].y, r[2 * q + 1].x, r[2 * q + 1].y);
+        }
+        return;
+    }
+    uint4* yo = static_cast<uint4*>(a.y) + t.at + (size_t)(c >> 3) * vp;
+    uint4 val[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        __nv_bfloat162 pk[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) pk[e] = __float22bfloat162_rn(r[4 * q + e]);
+        val[q] = *reinterpret_cast<uint4*>(pk);
+        if (t.valid) yo[q * vp] = val[q];
+    }
+    if (a.y_up) {
+        // The eight children on the doubled grid.  Lane i stores child i & 1 of lane i / 2 (then of lane
+        // 16 + i / 2), so that a warp's store covers whole 32-byte sectors: every lane storing its own
+        // children left half of each sector to another instruction.
+        const size_t row = 2 * (size_t)a.W + 2, plane = row * (2 * a.H + 2), vp_up = plane * (2 * a.D + 2);
+        uint4* yu = static_cast<uint4*>(a.y_up) + (size_t)(c >> 3) * vp_up;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int from = 16 * h + (lane >> 1);
+            const size_t at = (size_t)__shfl_sync(0xffffffffu, (unsigned long long)t.up, from) + (lane & 1);
+            const bool ok = __shfl_sync(0xffffffffu, (int)t.valid, from) != 0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint4 w;
+                w.x = __shfl_sync(0xffffffffu, val[q].x, from);
+                w.y = __shfl_sync(0xffffffffu, val[q].y, from);
+                w.z = __shfl_sync(0xffffffffu, val[q].z, from);
+                w.w = __shfl_sync(0xffffffffu, val[q].w, from);
+                if (ok) {
+                    uint4* d = yu + at + q * vp_up;
+                    d[0] = w;
+                    d[row] = w;
+                    d[plane] = w;
+                    d[plane + row] = w;
+                }
+            }
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, BrickPlan b) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // warp-uniform for the compiler too, so that the MMA warps' operands are
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int Cin = a.Cin, Cp = b.Cp, W = a.W, H = a.H, D = a.D;
     const int P = b.P, Yb = b.Yb;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem);  // [kPipeStages]
-    uint64_t* empty = full + kPipeStages;                 // [kPipeStages]
-    uint64_t* tfull = empty + kPipeStages;                // [2]
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);  // [kPipeStages][3 planes]
+    uint64_t* empty = full + 3 * kPipeStages;             // [kPipeStages][3 planes]
+    uint64_t* tfull = empty + 3 * kPipeStages;            // [2]
     uint64_t* tempty = tfull + 2;                         // [2]
     uint64_t* wfull = tempty + 2;                         // resident weights landed
-    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 128);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 132);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 160);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 164);
     const uint32_t s_stage0 = umma::smem_addr(smem) + kPipeHeader;
     if (warp == 0) {
         umma::tmem_alloc(slot, (uint32_t)b.tcols);
         umma::tmem_relinquish();
     }
     if (tid == 0) {
-        for (int s = 0; s < kPipeStages; ++s) {
+        for (int s = 0; s < 3 * kPipeStages; ++s) {
             umma::mbar_init(&full[s], 1);
-            umma::mbar_init(&empty[s], 2);  // one commit per MMA thread
+            umma::mbar_init(&empty[s], 2);  // one commit per MMA warp
         }
         for (int s = 0; s < 2; ++s) {
             umma::mbar_init(&tfull[s], 2);
-            umma::mbar_init(&tempty[s], kConvWorkerThreads);
+            umma::mbar_init(&tempty[s], 4 * b.tiles);  // one arrival per warp and tile
         }
         umma::mbar_init(wfull, 1);
         *abort_flag = 0;
@@ -345,290 +561,175 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
-    const uint32_t tbase = *slot;
+    const uint32_t tbase = __shfl_sync(0xffffffffu, *slot, 0);
     const int nchunk = Cin >> 4;
     const int acc_cols = b.tiles * Cp * (b.fold ? 3 : 1);
     const int tpr = W >> 7;                          // row tiles: M tiles per output row
     const uint32_t w_chunk = (uint32_t)(27 * Cp * 32);  // bytes of one chunk's weights
     const uint32_t s_wres = s_stage0 + (uint32_t)(kPipeStages * b.stage);
     const Pcg pg{D, H, W};
+    BrickItems t(b, D);
 
-    if (warp == kConvWorkers + 2) {
-        // producer warp: lane 0 waits for a free stage and posts the bytes it will receive, then
-        // lanes 0-5 issue the six brick runs and lane 6 the weight chunk (one thread can issue
-        // a bulk copy only every ~100 cycles, which made the copies the bottleneck of the
-        // 96-channel layer)
-        const int Gin = Cin >> 3;
-        int k = 0;
-        if (b.wres && lane == 0) {
-            umma::mbar_arrive_expect_tx(wfull, (uint32_t)nchunk * w_chunk);
-            umma::bulk_g2s(s_wres, a.wpk, (uint32_t)nchunk * w_chunk, wfull);
-        }
-        bool ok = true;
-        for (int item = blockIdx.x; ok && item < b.items; item += gridDim.x) {
-            const BrickItem t = brick_item(b, D, item);
-            const __nv_bfloat16* wpart = a.wpk + (size_t)t.part * nchunk * 27 * Cp * 16;
-            // one (channel group, plane) part of the brick: padded rows y0 .. y0+Yb-1, fewer in a
-            // last row block that passes H (the rows it leaves stale feed only outputs y >= H,
-            // which the epilogue drops)
-            const int rows = Yb < H + 2 - t.y0 ? Yb : H + 2 - t.y0;
-            const uint32_t run = (uint32_t)(rows * P * 16);
-            const uint32_t slot = (uint32_t)(Yb * P * 16);
-            for (int c = 0; c < nchunk; ++c, ++k) {
-                const int s = k % kPipeStages, u = k / kPipeStages;
-                bool got = true;
-                if (lane == 0 && u >= 1) got = pipe_wait(&empty[s], (uint32_t)(u - 1) & 1u, abort_flag);
-                if (!__shfl_sync(0xffffffffu, got, 0)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t st = s_stage0 + (uint32_t)(s * b.stage);
-                if (lane == 0) umma::mbar_arrive_expect_tx(&full[s], 6u * run + (b.wres ? 0u : w_chunk));
-                __syncwarp();
-                if (lane < 6) {  // rows y0-1 .. y0+Ty of plane z+zb-1, columns -1 .. W
-                    const int gg = lane / 3, zb = lane - 3 * gg;
-                    umma::bulk_g2s(st + 128u + (uint32_t)(gg * b.plane) + (uint32_t)zb * slot,
-                                   a.x + 8 * pg.unit(t.n, Gin, 2 * c + gg, t.z + zb - 1, t.y0 - 1, -1), run, &full[s]);
-                } else if (lane == 6 && !b.wres) {
-                    umma::bulk_g2s(st + (uint32_t)b.w_off, wpart + (size_t)c * 27 * Cp * 16, w_chunk, &full[s]);
+    if (warp >= kConvWorkers + 2) {
+        // copy warp of plane z - 1 + zb: its run of either channel group, its nine taps' weights
+        const int zb = warp - kConvWorkers - 2;
+        if (lane == 0) {
+            const size_t row = (size_t)P * 16, plane = (size_t)(H + 2) * row, group = pg.vp() * 16;
+            const unsigned char* src = reinterpret_cast<const unsigned char*>(a.x) + zb * plane;
+            const unsigned char* wsrc = reinterpret_cast<const unsigned char*>(a.wpk) + zb * (w_chunk / 3);
+            const uint32_t dst = s_stage0 + 128u + (uint32_t)(zb * Yb * P * 16);
+            const uint32_t wdst = s_stage0 + (uint32_t)b.w_off + (uint32_t)zb * (w_chunk / 3);
+            int k = 0, s = 0;
+            uint32_t par = 1;  // of the "empty" phase to wait for
+            if (b.wres && zb == 0) {
+                umma::mbar_arrive_expect_tx(wfull, (uint32_t)nchunk * w_chunk);
+                umma::bulk_g2s(s_wres, a.wpk, (uint32_t)nchunk * w_chunk, wfull);
+            }
+            bool ok = true;
+            for (; ok && t.left > 0; t.next(b, D)) {
+                const int y0 = t.yb * b.Ty;
+                // padded rows y0 .. y0+Yb-1 of the plane, fewer in a last row block that passes H (the
+                // rows it leaves stale feed only outputs y >= H, which the epilogue drops)
+                const uint32_t run = (uint32_t)((Yb < H + 2 - y0 ? Yb : H + 2 - y0) * P * 16);
+                const unsigned char* xs = src + ((size_t)t.n * (Cin >> 3) * group + (size_t)t.z * plane + (size_t)y0 * row);
+                const unsigned char* ws = wsrc + (size_t)t.part * nchunk * w_chunk;
+                for (int c = 0; c < nchunk; ++c, ++k) {
+                    uint64_t* f = &full[3 * s + zb];
+                    if (k >= kPipeStages && !(ok = pipe_wait(&empty[3 * s + zb], par, abort_flag))) break;
+                    const uint32_t st = (uint32_t)(s * b.stage);
+                    umma::mbar_arrive_expect_tx(f, 2u * run + (b.wres ? 0u : w_chunk / 3));
+                    umma::bulk_g2s(dst + st, xs, run, f);
+                    umma::bulk_g2s(dst + st + (uint32_t)b.plane, xs + group, run, f);
+                    if (!b.wres) umma::bulk_g2s(wdst + st, ws, w_chunk / 3, f);
+                    xs += 2 * group;
+                    ws += w_chunk;
+                    if (++s == kPipeStages) {
+                        s = 0;
+                        par ^= 1u;
+                    }
                 }
             }
-        }
-        if (lane == 0) {
-            // no copy may still be writing shared memory when the CTA exits: wait for the
-            // last kPipeStages chunks (earlier ones were consumed before their stage was reused)
+            // no copy may still be writing shared memory when the CTA exits: wait for this thread's last
+            // kPipeStages (earlier ones were consumed before their stage was reused)
             for (int kk = k > kPipeStages ? k - kPipeStages : 0; kk < k; ++kk)
-                umma::mbar_wait(&full[kk % kPipeStages], (uint32_t)(kk / kPipeStages) & 1u, kWaitCycles);
-            if (b.wres) umma::mbar_wait(wfull, 0u, kWaitCycles);
+                umma::mbar_wait(&full[3 * (kk % kPipeStages) + zb], (uint32_t)(kk / kPipeStages) & 1u, kWaitCycles);
+            if (b.wres && zb == 0) umma::mbar_wait(wfull, 0u, kWaitCycles);
         }
         __syncwarp();
     } else if (warp >= kConvWorkers) {
-        // two MMA threads (one thread can issue a tcgen05.mma only every ~65 cycles, two are
+        // two MMA warps (one thread can issue a tcgen05.mma only every ~65 cycles, two are
         // bound by the operand reads from shared memory): issuer iss takes the M tiles of its
         // parity, so each accumulator column range has one issuer
         const int iss = warp - kConvWorkers;
-        if (lane == 0) {
-            const uint32_t idesc = umma::idesc_bf16_f32(128, b.fold ? 3 * Cp : Cp);
-            int toff[27];  // tap (dz, dy, dx) -> brick position offset (dz Yb + dy) P + dx
-#pragma unroll
-            for (int t = 0; t < 27; ++t) toff[t] = ((t / 9 - 1) * Yb + ((t / 3) % 3 - 1)) * P + (t % 3 - 1);
-            int k = 0;
-            bool ok = !b.wres || pipe_wait(wfull, 0u, abort_flag);
-            for (int item = blockIdx.x, j = 0; ok && item < b.items; item += gridDim.x, ++j) {
-                const int acc = j % b.nacc, v = j / b.nacc;
-                if (v >= 1 && !pipe_wait(&tempty[acc], (uint32_t)(v - 1) & 1u, abort_flag)) break;
-                umma::fence_after_sync();
-                const uint32_t dacc = tbase + (uint32_t)(acc * acc_cols);
-                for (int c = 0; c < nchunk; ++c, ++k) {
-                    const int s = k % kPipeStages, u = k / kPipeStages;
-                    if (!pipe_wait(&full[s], (uint32_t)u & 1u, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    umma::fence_after_sync();
-                    const uint32_t st = s_stage0 + (uint32_t)(s * b.stage);
-                    const uint64_t a0 = umma::smem_desc(st + 128u, (uint32_t)b.plane, 128);
-                    const uint64_t b0 = umma::smem_desc(
-                        b.wres ? s_wres + (uint32_t)c * w_chunk : st + (uint32_t)b.w_off, 128, 256);
-                    const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32);
-                    const uint32_t b_lo = (uint32_t)b0, b_hi = (uint32_t)(b0 >> 32);
-                    const uint32_t first = c > 0 ? 1u : 0u;
-                    const bool rt = b.rowtile != 0;
-                    if (b.fold) {
-                        switch (b.tiles) {
-#define SDE_CONV_FOLD(T)                                                                             \
-    case T:                                                                                          \
-        if (iss) conv_chunk_mma_fold<T, 1>(dacc, a_lo, a_hi, b_lo, b_hi, idesc, Cp, toff, P, Yb, first); \
-        else conv_chunk_mma_fold<T, 0>(dacc, a_lo, a_hi, b_lo, b_hi, idesc, Cp, toff, P, Yb, first); \
+        IssueArgs g;
+        g.full = full;
+        g.empty = empty;
+        g.tfull = tfull;
+        g.tempty = tempty;
+        g.abort_flag = abort_flag;
+        g.a0 = umma::smem_desc(s_stage0 + 128u, (uint32_t)b.plane, 128);
+        g.b0 = umma::smem_desc(b.wres ? s_wres : s_stage0 + (uint32_t)b.w_off, 128, 256);
+        g.tbase = tbase;
+        g.idesc = umma::idesc_bf16_f32(128, b.fold ? 3 * Cp : Cp);
+        g.leader = umma::elect_one();
+        g.items = t.left;
+        g.nchunk = nchunk;
+        g.Cp = Cp;
+        g.tpr = tpr;
+        if (__all_sync(0xffffffffu, !b.wres || pipe_wait(wfull, 0u, abort_flag))) {
+            switch (b.tiles + (b.fold ? 100 : 0)) {
+#define SDE_CONV_ISSUE(F, T)                        \
+    case (F ? 100 : 0) + T:                         \
+        if (iss) conv_issue<F, T, 1>(b, g);         \
+        else conv_issue<F, T, 0>(b, g);             \
         break;
-                            SDE_CONV_FOLD(1)
-                            SDE_CONV_FOLD(2)
-                            SDE_CONV_FOLD(3)
-                            SDE_CONV_FOLD(4)
-#undef SDE_CONV_FOLD
-                            default:  // the plan keeps folded items to <= 4 tiles
-                                *abort_flag = 1;
-                        }
-                    } else {
-                        switch (b.tiles) {
-#define SDE_CONV_TILES(T)                                                                          \
-    case T:                                                                                        \
-        if (iss) conv_chunk_mma<T, 1>(dacc, a_lo, a_hi, b_lo, b_hi, idesc, Cp, toff, rt, P, Yb, tpr, first); \
-        else conv_chunk_mma<T, 0>(dacc, a_lo, a_hi, b_lo, b_hi, idesc, Cp, toff, rt, P, Yb, tpr, first); \
-        break;
-                            SDE_CONV_TILES(1)
-                            SDE_CONV_TILES(2)
-                            SDE_CONV_TILES(3)
-                            SDE_CONV_TILES(4)
-                            SDE_CONV_TILES(5)
-                            SDE_CONV_TILES(6)
-                            SDE_CONV_TILES(7)
-                            SDE_CONV_TILES(8)
-#undef SDE_CONV_TILES
-                            default:  // the plan keeps items to <= 8 tiles
-                                *abort_flag = 1;
-                        }
-                    }
-                    umma::mma_commit(&empty[s]);
-                }
-                if (ok) umma::mma_commit(&tfull[acc]);
+                SDE_CONV_ISSUE(true, 1)
+                SDE_CONV_ISSUE(true, 2)
+                SDE_CONV_ISSUE(true, 3)
+                SDE_CONV_ISSUE(true, 4)
+                SDE_CONV_ISSUE(false, 1)
+                SDE_CONV_ISSUE(false, 2)
+                SDE_CONV_ISSUE(false, 3)
+                SDE_CONV_ISSUE(false, 4)
+                SDE_CONV_ISSUE(false, 5)
+                SDE_CONV_ISSUE(false, 6)
+                SDE_CONV_ISSUE(false, 7)
+                SDE_CONV_ISSUE(false, 8)
+#undef SDE_CONV_ISSUE
+                default:  // the plan keeps items to <= 8 tiles, folded ones to <= 4
+                    *abort_flag = 1;
             }
         }
         __syncwarp();
     } else {
-        // epilogue: thread 0 polls each barrier and the outcome is shared through a
-        // named-barrier vote, so control flow stays uniform and a timeout ends all warps
-        bool ok = true;
-        auto worker_wait = [&](uint64_t* m, uint32_t parity) {
-            bool done = true;
-            if (tid == 0) done = pipe_wait(m, parity, abort_flag);
-            return workers_all<kConvWorkerThreads>(done);
-        };
+        // epilogue: the CTA's M tiles, all items' in order, go round the groups.  Each warp waits for its
+        // tile's accumulator by itself; after a timeout it goes on through its tiles without storing,
+        // so that the group's barriers still meet.
         const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. + 31
-        const int grp = warp >> 2;     // warps 0-3 take the even tiles of an item, 4-7 the odd ones
+        const int grp = warp >> 2;
+        const size_t vp = pg.vp();
         const int Gy = a.y_cstride >> 3;
-        // fold: per group two buffers (alternate tiles) of [lane quarter][Cp] column values at
-        // the quarter's edges: D[x = 32 quarter + 31][co] and D[x = 32 quarter][2 Cp + co]
-        float* xbuf = reinterpret_cast<float*>(smem + b.xch);
+        // fold: per group two buffers (alternate columns; one where Cp = 16 leaves room for no more) of
+        // [2][lane quarter][16] values at the quarters' edges: D[x = 32 quarter + 31][co] and
+        // D[x = 32 quarter][2 Cp + co]
+        const bool one_buffer = Cp < 32;
+        float* xbuf = reinterpret_cast<float*>(smem + b.xch) + grp * (one_buffer ? 128 : 256);
         int par = 0;
-        for (int item = blockIdx.x, j = 0; ok && item < b.items; item += gridDim.x, ++j) {
-            const int acc = j % b.nacc, v = j / b.nacc;
-            if (!worker_wait(&tfull[acc], (uint32_t)v & 1u)) {
-                ok = false;
-                break;
+        bool ok = true;
+        uint32_t acc_par = 0;
+        int acc = 0, m = grp;
+        while (t.left > 0) {
+            if (m >= b.tiles) {  // on to the next item
+                m -= b.tiles;
+                t.next(b, D);
+                if (++acc == b.nacc) {
+                    acc = 0;
+                    acc_par ^= 1u;
+                }
+                continue;
             }
+            if (lane == 0) ok = ok && pipe_wait(&tfull[acc], acc_par, abort_flag);
+            ok = __shfl_sync(0xffffffffu, ok, 0);
             umma::fence_after_sync();
-            const BrickItem t = brick_item(b, D, item);
-            const int cbase = t.part * Cp;
-            const uint32_t trow = tbase + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(acc * acc_cols);
-            for (int m = warp >> 2; m < b.tiles; m += kConvWorkers / 4) {
-                int yy, xx;
-                bool valid = true;
-                if (b.rowtile) {
-                    yy = t.y0 + m / tpr;
-                    xx = 128 * (m % tpr) + 32 * quarter + lane;
-                    valid = yy < H;
-                } else {
-                    const int q = P + 128 * m + 32 * quarter + lane;  // position in brick plane zb = 1
-                    const int yb = q / P, xp = q - yb * P;
-                    yy = t.y0 + yb - 1;
-                    xx = xp - 1;
-                    valid = yb >= 1 && yb <= b.Ty && xp >= 1 && xp <= W && yy < H;
-                }
-                // fold: out[x] = D[x-1][co] + D[x][Cp + co] + D[x+1][2 Cp + co]; x - 1 and x + 1 of the
-                // quarter's edge lanes belong to the neighbouring quarter (another warp of the group),
-                // x = -1 and x = 128 are padding (their D is zero).  Columns move 16 at a time, all
-                // loads of a chunk in flight before one wait.
-                const uint32_t tcol = trow + (uint32_t)(m * Cp * (b.fold ? 3 : 1));
-                float* xlo = xbuf + (size_t)((grp * 2 + par) * 2) * 4 * Cp;
-                float* xhi = xlo + 4 * Cp;
-                for (int c = 0; c < Cp; c += 16) {
-                    uint32_t v[16];
-                    __syncwarp();
-                    if (b.fold) {
-                        uint32_t lo[16], hi[16];
-                        umma::tmem_ld16_nowait(tcol + (uint32_t)c, lo);
-                        umma::tmem_ld16_nowait(tcol + (uint32_t)(Cp + c), v);
-                        umma::tmem_ld16_nowait(tcol + (uint32_t)(2 * Cp + c), hi);
-                        umma::tmem_wait_ld16(lo);
-                        umma::tmem_touch16(v);
-                        umma::tmem_touch16(hi);
-                        // edge lanes publish their 16 values with four 16-byte stores
-                        if (lane == 31 || lane == 0) {
-                            uint4* dst = reinterpret_cast<uint4*>((lane == 31 ? xlo : xhi) + quarter * Cp + c);
-                            const uint32_t* src = lane == 31 ? lo : hi;
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4)
-                                dst[q4] = make_uint4(src[4 * q4], src[4 * q4 + 1], src[4 * q4 + 2], src[4 * q4 + 3]);
-                        }
-                        uint32_t l[16], r[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            l[e] = __shfl_up_sync(0xffffffffu, lo[e], 1);
-                            r[e] = __shfl_down_sync(0xffffffffu, hi[e], 1);
-                        }
-                        group_sync(2 + grp);
-                        if (lane == 0 || lane == 31) {
-                            const bool left = lane == 0;
-                            const bool edge = left ? quarter == 0 : quarter == 3;  // padding column
-                            const int nq = left ? (quarter > 0 ? quarter - 1 : 0) : (quarter < 3 ? quarter + 1 : 3);
-                            const uint4* src = reinterpret_cast<const uint4*>((left ? xlo : xhi) + nq * Cp + c);
-                            uint32_t* dst = left ? l : r;
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                const uint4 w = edge ? make_uint4(0u, 0u, 0u, 0u) : src[q4];
-                                dst[4 * q4] = w.x;
-                                dst[4 * q4 + 1] = w.y;
-                                dst[4 * q4 + 2] = w.z;
-                                dst[4 * q4 + 3] = w.w;
-                            }
-                        }
-#pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            v[e] = __float_as_uint(__uint_as_float(v[e]) + (__uint_as_float(l[e]) + __uint_as_float(r[e])));
-                    } else {
-                        umma::tmem_ld16_nowait(tcol + (uint32_t)c, v);
-                        umma::tmem_wait_ld16(v);
-                    }
-                    if (valid) {
-                        float rr[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) rr[e] = __uint_as_float(v[e]);
-                        if (a.bias) {
-                            const float4* bq = reinterpret_cast<const float4*>(a.bias + cbase + c);
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                const float4 bb = __ldg(bq + q4);
-                                rr[4 * q4] += bb.x;
-                                rr[4 * q4 + 1] += bb.y;
-                                rr[4 * q4 + 2] += bb.z;
-                                rr[4 * q4 + 3] += bb.w;
-                            }
-                        }
-                        if (a.relu)
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) rr[e] = rr[e] > 0.f ? rr[e] : a.slope * rr[e];
-                        if (a.y_fp32) {
-                            const size_t vox = (size_t)t.n * a.nvox + ((size_t)t.z * H + yy) * W + xx;
-                            if (a.y_keep) {  // leading channels only (the first chunk of part 0)
-                                if (cbase + c == 0)
-#pragma unroll
-                                    for (int e = 0; e < 16; ++e)  // constant indices keep rr in registers
-                                        if (e < a.y_keep) static_cast<float*>(a.y)[vox * a.y_keep + e] = rr[e];
-                            } else {
-                                float4* yo = reinterpret_cast<float4*>(static_cast<float*>(a.y) + vox * a.y_cstride +
-                                                                       a.y_coffset + cbase + c);
-                                for (int q4 = 0; q4 < 4; ++q4)
-                                    yo[q4] = make_float4(rr[4 * q4], rr[4 * q4 + 1], rr[4 * q4 + 2], rr[4 * q4 + 3]);
-                            }
-                        } else {
-                            for (int h = 0; h < 2; ++h) {
-                                __nv_bfloat162 pk[4];
-                                for (int e = 0; e < 4; ++e)
-                                    pk[e] = __floats2bfloat162_rn(rr[8 * h + 2 * e], rr[8 * h + 2 * e + 1]);
-                                const int gy = (a.y_coffset + cbase + c + 8 * h) >> 3;
-                                __nv_bfloat16* yo =
-                                    static_cast<__nv_bfloat16*>(a.y) + 8 * pg.unit(t.n, Gy, gy, t.z, yy, xx);
-                                const uint4 val = *reinterpret_cast<uint4*>(pk);
-                                *reinterpret_cast<uint4*>(yo) = val;
-                                if (a.y_up) {  // the eight children on the doubled grid
-                                    const Pcg pf{2 * D, 2 * H, 2 * W};
-                                    const int gu = (a.y_up_coffset + cbase + c + 8 * h) >> 3;
-                                    __nv_bfloat16* yu = static_cast<__nv_bfloat16*>(a.y_up);
-#pragma unroll
-                                    for (int d = 0; d < 8; ++d)
-                                        *reinterpret_cast<uint4*>(
-                                            yu + 8 * pf.unit(t.n, a.y_up_cstride >> 3, gu, 2 * t.z + (d >> 2),
-                                                             2 * yy + ((d >> 1) & 1), 2 * xx + (d & 1))) = val;
-                                }
-                            }
-                        }
-                    }
-                }
-                par ^= 1;
+            const int y0 = t.yb * b.Ty, cbase = t.part * Cp;
+            int yy, xx;
+            bool valid;
+            if (b.rowtile) {
+                yy = y0 + m / tpr;
+                xx = 128 * (m % tpr) + 32 * quarter + lane;
+                valid = yy < H;
+            } else {
+                const int q = P + 128 * m + 32 * quarter + lane;  // position in brick plane zb = 1
+                const int yb = q / P, xp = q - yb * P;
+                yy = y0 + yb - 1;
+                xx = xp - 1;
+                valid = yb >= 1 && yb <= b.Ty && xp >= 1 && xp <= W && yy < H;
+            }
+            TileVoxel tv;
+            tv.valid = valid && ok;
+            if (a.y_fp32)
+                tv.at = (size_t)t.n * a.nvox + ((size_t)t.z * H + yy) * W + xx;
+            else
+                tv.at = pg.unit(t.n, Gy, (a.y_coffset + cbase) >> 3, t.z, yy, xx);
+            if (a.y_up)
+                tv.up = Pcg{2 * D, 2 * H, 2 * W}.unit(t.n, a.y_up_cstride >> 3, (a.y_up_coffset + cbase) >> 3, 2 * t.z,
+                                                     2 * yy, 2 * xx);
+            const uint32_t tcol = tbase + ((uint32_t)(32 * quarter) << 16) +
+                                  (uint32_t)(acc * acc_cols + m * Cp * (b.fold ? 3 : 1));
+            for (int c = 0; c < Cp; c += 16) {
+                float2 r[8];
+                __syncwarp();
+                if (b.fold)
+                    tile_columns<true>(tcol + (uint32_t)c, Cp, xbuf + 128 * par, one_buffer, quarter, lane, 1 + grp, r);
+                else
+                    tile_columns<false>(tcol + (uint32_t)c, Cp, nullptr, false, quarter, lane, 0, r);
+                if (!one_buffer) par ^= 1;
+                store_columns(a, tv, cbase, c, lane, vp, r);
             }
             umma::fence_before_sync();
-            umma::mbar_arrive(&tempty[acc]);
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(&tempty[acc]);
+            m += kConvGroups;
         }
     }
     umma::fence_before_sync();
