@@ -773,28 +773,28 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 //
 // Bound by the MMAs (N / 2 cycles each: the dense rate, a quarter of M used by 32 channels of the
 // long sums, three quarters of the short ones).  Before, one MMA a tap with 16 or 32 channels in N
-// and the x brick loaded once per tap group: 32 -> 32 channels on 192x128x128 0.915 -> 0.435 ms (long
-// order, 87 % of the MMAs' time), 64 -> 96 on 66x54x128 0.316 -> 0.149 ms (short order).
+// and the x brick loaded once per tap group: 32 -> 32 channels on 192x128x128 0.915 -> 0.398 ms (long
+// order: 0.33 ms of MMAs), 64 -> 96 on 66x54x128 0.316 -> 0.149 ms (short order).
 // ----------------------------------------------------------------------------
 constexpr int kRingMaxX = 12, kRingMaxD = 4, kRingCopyWarps = 8, kRingWarps = kRingCopyWarps + 3;
 
-// The MMAs of one item, offset and run of planes.  Unrolled, because address arithmetic between
-// two MMAs of one thread costs more than the MMA.
-__device__ __forceinline__ void ring_mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, int kst, uint32_t first) {
-    const uint32_t a_hi = (uint32_t)(ad >> 32), b_hi = (uint32_t)(bd >> 32);
-    uint32_t a_lo = (uint32_t)ad, b_lo = (uint32_t)bd;
-    umma::mma_bf16_lohi(d, a_lo, a_hi, b_lo, b_hi, idesc, first);
+// The MMAs of one item, offset and run of planes, issued by a whole warp's leader.  Unrolled,
+// because address arithmetic between two MMAs of one warp costs more than the MMA.
+__device__ __forceinline__ void ring_mma(uint32_t leader, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                         uint32_t b_hi, uint32_t idesc, int kst, uint32_t first) {
+    umma::mma_bf16_warp(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, first);
     int ks = 1;
     for (; ks + 4 <= kst; ks += 4) {
 #pragma unroll
-        for (int u = 1; u <= 4; ++u) umma::mma_bf16_lohi(d, a_lo + 16 * u, a_hi, b_lo + 16 * u, b_hi, idesc, 1u);
+        for (int u = 1; u <= 4; ++u)
+            umma::mma_bf16_warp(leader, d, a_lo + 16 * u, a_hi, b_lo + 16 * u, b_hi, idesc, 1u);
         a_lo += 64;
         b_lo += 64;
     }
     for (; ks < kst; ++ks) {
         a_lo += 16;
         b_lo += 16;
-        umma::mma_bf16_lohi(d, a_lo, a_hi, b_lo, b_hi, idesc, 1u);
+        umma::mma_bf16_warp(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, 1u);
     }
 }
 
@@ -849,11 +849,12 @@ struct RingSlot {
 
 __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, WgradRing b) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // warp-uniform for the compiler too, so that the issuers' operands are
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int Cin = a.Cin, Cout = a.Cout, W = a.W, H = a.H, D = a.D, Yb = b.Ty + 2;
     uint64_t* fullx = reinterpret_cast<uint64_t*>(smem);  // [XS] plane landed
     uint64_t* emptyx = fullx + kRingMaxX;                  // [XS] no later MMA reads the plane
-    uint64_t* fulld = emptyx + kRingMaxX;                  // [DS] dy rows landed
+    uint64_t* fulld = emptyx + kRingMaxX;                  // [DS] dy rows landed (long order: planes too)
     uint64_t* emptyd = fulld + kRingMaxD;                  // [DS] item's MMAs finished
     uint64_t* dfull = emptyd + kRingMaxD;                  // all MMAs of the CTA finished
     uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 320);
@@ -884,7 +885,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
-    const uint32_t tbase = *slot;
+    const uint32_t tbase = __shfl_sync(0xffffffffu, *slot, 0);
     const int N = 8 * b.ngr;  // columns of an accumulator
     RingItems it(b, D);
     const bool any = it.left > 0;
@@ -908,88 +909,125 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
             }
             const unsigned char* xsrc =
                 reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.gpp, -1, -1, -1));
-            RingSlot sd, sx;
-            int j = 0, turn = nd, fresh = 3;  // fresh: planes this item brings; turn: copies go round the warps
-            size_t planes = 0;
+            RingSlot sd;
+            int j = 0;
             bool ok = true;
-            for (; it.left > 0; ++j) {
-                if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
-                const size_t at = (size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16);
-                if (warp == 0) umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
+            if (b.order) {
+                // every item brings its three planes, on the dy slot's barrier; warp w's plane copy is
+                // group w % gpp of plane w / gpp
+                const int q = warp % b.gpp, f = warp / b.gpp;
+                const unsigned char* xs = xsrc + f * plane + q * vp;
+                const uint32_t xdst = s_x + (uint32_t)(f * b.xslot) + (uint32_t)q * xrun;
+                const uint32_t bytes = (uint32_t)(nd * b.drun) + 3u * (uint32_t)b.gpp * xrun;
+                for (; it.left > 0; ++j) {
+                    if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
+                    uint64_t* full = &fulld[sd.i];
+                    const size_t at = (size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16);
+                    if (warp == 0) umma::mbar_arrive_expect_tx(full, bytes);
+                    if (f < 3)
+                        umma::bulk_g2s(xdst + (uint32_t)(3 * sd.i * b.xslot), xs + at + (size_t)it.n * gx * vp, xrun, full);
 #pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    if (mine[e])
-                        umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
-                                       (uint32_t)b.drun, &fulld[sd.i]);
-                const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
-                for (int f = 0; f < fresh; ++f, ++planes) {
-                    // in the long order a plane slot goes with the dy slot that was waited for
-                    if (!b.order && planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag)))
-                        break;
-                    if (warp == 0) umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
-                    for (int q = 0; q < b.gpp; ++q, ++turn)
-                        if (turn % kRingCopyWarps == warp)
-                            umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
-                                           &fullx[sx.i]);
-                    xat += plane;
-                    sx.advance(b.XS);
+                    for (int e = 0; e < 2; ++e)
+                        if (mine[e])
+                            umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
+                                           (uint32_t)b.drun, full);
+                    sd.advance(b.DS);
+                    it.next(b, D);
                 }
-                if (!ok) break;
-                fresh = it.shares(b, D) ? 1 : 3;
-                sd.advance(b.DS);
-                it.next(b, D);
+            } else {
+                RingSlot sx;
+                int turn = nd, fresh = 3;  // fresh: planes this item brings; turn: copies go round the warps
+                size_t planes = 0;
+                for (; it.left > 0; ++j) {
+                    if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
+                    const size_t at = (size_t)it.z * plane + (size_t)it.yb * (b.P * 16);
+                    if (warp == 0) umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        if (mine[e])
+                            umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
+                                           (uint32_t)b.drun, &fulld[sd.i]);
+                    const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
+                    for (int f = 0; f < fresh; ++f, ++planes) {
+                        if (planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag))) break;
+                        if (warp == 0) umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
+                        for (int q = 0; q < b.gpp; ++q, ++turn)
+                            if (turn % kRingCopyWarps == warp)
+                                umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
+                                               &fullx[sx.i]);
+                        xat += plane;
+                        sx.advance(b.XS);
+                    }
+                    if (!ok) break;
+                    fresh = it.shares(b, D) ? 1 : 3;
+                    sd.advance(b.DS);
+                    it.next(b, D);
+                }
             }
             if (!ok) *abort_flag = 1;  // an expected copy may not come: no one may wait for it
         }
         __syncwarp();
     } else if (warp - kRingCopyWarps < b.nt) {  // issuer of offset t
         const int t = warp - kRingCopyWarps;
-        if (lane == 0) {
-            const uint32_t d = tbase + (uint32_t)(t * N);
-            // leading byte offset = next 8 positions (K); stride = next 8 channels of dy, next row,
-            // 8-channel group or plane of x
-            const uint64_t a0 = umma::smem_desc(s_d, 128, (uint32_t)b.ra);
-            const uint64_t b0 = umma::smem_desc((uint32_t)((int)s_x + 16 * (b.xoff + t)), 128, (uint32_t)b.P * 16u);
-            const uint32_t idesc = umma::idesc_bf16_f32(128, N, 1, 1);
+        const uint32_t leader = umma::elect_one(), d = tbase + (uint32_t)(t * N);
+        // leading byte offset = next 8 positions (K); stride = next 8 channels of dy, next row,
+        // 8-channel group or plane of x; descriptors step by their start field, in 16-byte units
+        const uint64_t a0 = umma::smem_desc(s_d, 128, (uint32_t)b.ra);
+        const uint64_t b0 = umma::smem_desc((uint32_t)((int)s_x + 16 * (b.xoff + t)), 128, (uint32_t)b.P * 16u);
+        const uint32_t a_hi = (uint32_t)(a0 >> 32), b_hi = (uint32_t)(b0 >> 32);
+        const uint32_t idesc = umma::idesc_bf16_f32(128, N, 1, 1);
+        const uint32_t dstep = (uint32_t)b.dslot >> 4, xstep = (uint32_t)b.xslot >> 4;
+        RingSlot sd;
+        uint32_t accum = 0, a_lo = (uint32_t)a0;
+        bool ok = true;
+        if (b.order) {
+            uint32_t b_lo = (uint32_t)b0;
+            for (int left = it.left; left > 0; --left) {
+                ok = pipe_wait(&fulld[sd.i], sd.par, abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) break;
+                umma::fence_after_sync();
+                ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, accum);
+                accum = 1;
+                umma::mma_commit_warp(leader, &emptyd[sd.i]);
+                sd.advance(b.DS);
+                a_lo = sd.i ? a_lo + dstep : (uint32_t)a0;
+                b_lo = sd.i ? b_lo + 3 * xstep : (uint32_t)b0;
+            }
+        } else {
             const int gp = b.gpp * Yb;  // row groups of a plane
-            RingSlot sd, seen;
+            RingSlot seen;
             int k = 0, fresh = 3;  // k: slot of the z-1 plane
-            uint32_t accum = 0;
-            bool ok = true;
             while (it.left > 0) {
                 for (int f = 0; ok && f < fresh; ++f) {
                     ok = pipe_wait(&fullx[seen.i], seen.par, abort_flag);
                     seen.advance(b.XS);
                 }
                 ok = ok && pipe_wait(&fulld[sd.i], sd.par, abort_flag);
-                if (!ok) break;
+                if (!__all_sync(0xffffffffu, ok)) break;
                 umma::fence_after_sync();
-                // descriptors step by their start field, in 16-byte units
-                const uint64_t ad = a0 + (uint32_t)(sd.i * (b.dslot >> 4)), bd = b0 + (uint32_t)(k * (b.xslot >> 4));
+                const uint32_t b_lo = (uint32_t)b0 + (uint32_t)k * xstep;
                 const int run = b.XS - k;  // planes before the ring wraps
                 if (run >= 3) {
-                    ring_mma(d, ad, bd, idesc, b.kst, accum);
+                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, accum);
                 } else {
                     const int n1 = run * gp;
-                    ring_mma(d, ad, bd, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, accum);
-                    ring_mma(d + (uint32_t)(8 * n1), ad, b0, umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, accum);
+                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, accum);
+                    ring_mma(leader, d + (uint32_t)(8 * n1), a_lo, a_hi, (uint32_t)b0, b_hi,
+                             umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, accum);
                 }
                 accum = 1;
-                umma::mma_commit(&emptyd[sd.i]);
+                umma::mma_commit_warp(leader, &emptyd[sd.i]);
                 sd.advance(b.DS);
+                a_lo = sd.i ? a_lo + dstep : (uint32_t)a0;
                 fresh = it.shares(b, D) ? 1 : 3;
-                if (b.order) {
-                    k = k + 3 < b.XS ? k + 3 : 0;
-                } else {
-                    for (int f = 0; f < fresh; ++f) {
-                        umma::mma_commit(&emptyx[k]);
-                        k = k + 1 < b.XS ? k + 1 : 0;
-                    }
+                for (int f = 0; f < fresh; ++f) {
+                    umma::mma_commit_warp(leader, &emptyx[k]);
+                    k = k + 1 < b.XS ? k + 1 : 0;
                 }
                 it.next(b, D);
             }
-            if (ok) umma::mma_commit(dfull);
         }
+        if (ok) umma::mma_commit_warp(leader, dfull);
         __syncwarp();
     }
     __syncthreads();
