@@ -236,9 +236,8 @@ __device__ __forceinline__ bool pipe_wait(uint64_t* m, uint32_t parity, volatile
 }
 
 // Epilogue warps of the brick convolution, groups of four that cover a tile's 128 lanes (warp &
-// 3: the tensor-memory lane quarter); the two MMA warps and the copy warps follow them.  32 -> 32
-// channels on 192x128x128: two groups 175 us, three 165, four 167.
-constexpr int kConvGroups = 3;
+// 3: the tensor-memory lane quarter); the two MMA warps and the copy warps follow them.
+constexpr int kConvGroups = 4;
 constexpr int kConvWorkers = 4 * kConvGroups;
 constexpr int kConvCopyWarps = 3;  // one per brick plane
 constexpr int kConvThreads = 32 * (kConvWorkers + 2 + kConvCopyWarps);
@@ -434,18 +433,17 @@ __device__ __forceinline__ void tile_columns(uint32_t tcol, int Cp, float* xch, 
     }
 }
 
-// Where a tile's lane writes: the 16-byte unit of its voxel in the part's first channel group of y
-// (FP32 output: its voxel index), that of its first child on the doubled grid, and whether it
-// is an output voxel.
+// Where a lane writes sixteen channels: the 16-byte unit of its voxel in the first of the two
+// channel groups of y (FP32 output: its voxel index), that of its first child on the doubled
+// grid, and whether it is an output voxel.
 struct TileVoxel {
     size_t at, up;
     bool valid;
 };
 
-// Bias, leaky ReLU and the stores of the sixteen channels from cbase + c on (tile_columns in r).
-__device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel& t, int cbase, int c, int lane, size_t vp,
+// Bias, leaky ReLU and the stores of the sixteen channels from ch on (tile_columns in r).
+__device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel& t, int ch, int lane, size_t vp,
                                               float2 (&r)[8]) {
-    const int ch = cbase + c;
     if (a.bias) {
         const float4* bq = reinterpret_cast<const float4*>(a.bias + ch);
 #pragma unroll
@@ -488,7 +486,7 @@ __device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel
         }
         return;
     }
-    uint4* yo = static_cast<uint4*>(a.y) + t.at + (size_t)(c >> 3) * vp;
+    uint4* yo = static_cast<uint4*>(a.y) + t.at;
     uint4 val[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -503,7 +501,7 @@ __device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel
         // 16 + i / 2), so that a warp's store covers whole 32-byte sectors: every lane storing its own
         // children left half of each sector to another instruction.
         const size_t row = 2 * (size_t)a.W + 2, plane = row * (2 * a.H + 2), vp_up = plane * (2 * a.D + 2);
-        uint4* yu = static_cast<uint4*>(a.y_up) + (size_t)(c >> 3) * vp_up;
+        uint4* yu = static_cast<uint4*>(a.y_up);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int from = 16 * h + (lane >> 1);
@@ -553,7 +551,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
         }
         for (int s = 0; s < 2; ++s) {
             umma::mbar_init(&tfull[s], 2);
-            umma::mbar_init(&tempty[s], 4 * b.tiles);  // one arrival per warp and tile
+            umma::mbar_init(&tempty[s], 4 * b.tiles * (Cp >> 4));  // one arrival per warp and block of columns
         }
         umma::mbar_init(wfull, 1);
         *abort_flag = 0;
@@ -662,14 +660,14 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
         }
         __syncwarp();
     } else {
-        // epilogue: the CTA's M tiles, all items' in order, go round the groups.  Each warp waits for its
-        // tile's accumulator by itself; after a timeout it goes on through its tiles without storing,
-        // so that the group's barriers still meet.
+        // epilogue: the blocks of sixteen columns of the CTA's M tiles, all items' in order, go round
+        // the groups.  Each warp waits for its tile's accumulator by itself; after a timeout it goes on
+        // through its blocks without storing, so that the group's barriers still meet.
         const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. + 31
-        const int grp = warp >> 2;
+        const int grp = warp >> 2, blocks = Cp >> 4;
         const size_t vp = pg.vp();
         const int Gy = a.y_cstride >> 3;
-        // fold: per group two buffers (alternate columns; one where Cp = 16 leaves room for no more) of
+        // fold: per group two buffers (used in turn; one where Cp = 16 leaves room for no more) of
         // [2][lane quarter][16] values at the quarters' edges: D[x = 32 quarter + 31][co] and
         // D[x = 32 quarter][2 Cp + co]
         const bool one_buffer = Cp < 32;
@@ -677,10 +675,12 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
         int par = 0;
         bool ok = true;
         uint32_t acc_par = 0;
-        int acc = 0, m = grp;
+        int acc = 0, m = 0, blk = grp;
         while (t.left > 0) {
-            if (m >= b.tiles) {  // on to the next item
-                m -= b.tiles;
+            if (blk >= blocks) {  // on to the next tile
+                blk -= blocks;
+                if (++m < b.tiles) continue;
+                m = 0;
                 t.next(b, D);
                 if (++acc == b.nacc) {
                     acc = 0;
@@ -691,12 +691,25 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
             if (lane == 0) ok = ok && pipe_wait(&tfull[acc], acc_par, abort_flag);
             ok = __shfl_sync(0xffffffffu, ok, 0);
             umma::fence_after_sync();
-            const int y0 = t.yb * b.Ty, cbase = t.part * Cp;
+            const int c = 16 * blk, ch = t.part * Cp + c;
+            const uint32_t tcol = tbase + ((uint32_t)(32 * quarter) << 16) +
+                                  (uint32_t)(acc * acc_cols + m * Cp * (b.fold ? 3 : 1) + c);
+            float2 r[8];
+            __syncwarp();
+            if (b.fold)
+                tile_columns<true>(tcol, Cp, xbuf + 128 * par, one_buffer, quarter, lane, 1 + grp, r);
+            else
+                tile_columns<false>(tcol, Cp, nullptr, false, quarter, lane, 0, r);
+            if (!one_buffer) par ^= 1;
+            umma::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(&tempty[acc]);  // the columns are in registers
+            const int y0 = t.yb * b.Ty;
             int yy, xx;
             bool valid;
             if (b.rowtile) {
-                yy = y0 + m / tpr;
-                xx = 128 * (m % tpr) + 32 * quarter + lane;
+                yy = y0 + (tpr == 2 ? m >> 1 : m);
+                xx = (tpr == 2 ? 128 * (m & 1) : 0) + 32 * quarter + lane;
                 valid = yy < H;
             } else {
                 const int q = P + 128 * m + 32 * quarter + lane;  // position in brick plane zb = 1
@@ -710,26 +723,12 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
             if (a.y_fp32)
                 tv.at = (size_t)t.n * a.nvox + ((size_t)t.z * H + yy) * W + xx;
             else
-                tv.at = pg.unit(t.n, Gy, (a.y_coffset + cbase) >> 3, t.z, yy, xx);
+                tv.at = pg.unit(t.n, Gy, (a.y_coffset + ch) >> 3, t.z, yy, xx);
             if (a.y_up)
-                tv.up = Pcg{2 * D, 2 * H, 2 * W}.unit(t.n, a.y_up_cstride >> 3, (a.y_up_coffset + cbase) >> 3, 2 * t.z,
-                                                     2 * yy, 2 * xx);
-            const uint32_t tcol = tbase + ((uint32_t)(32 * quarter) << 16) +
-                                  (uint32_t)(acc * acc_cols + m * Cp * (b.fold ? 3 : 1));
-            for (int c = 0; c < Cp; c += 16) {
-                float2 r[8];
-                __syncwarp();
-                if (b.fold)
-                    tile_columns<true>(tcol + (uint32_t)c, Cp, xbuf + 128 * par, one_buffer, quarter, lane, 1 + grp, r);
-                else
-                    tile_columns<false>(tcol + (uint32_t)c, Cp, nullptr, false, quarter, lane, 0, r);
-                if (!one_buffer) par ^= 1;
-                store_columns(a, tv, cbase, c, lane, vp, r);
-            }
-            umma::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) umma::mbar_arrive(&tempty[acc]);
-            m += kConvGroups;
+                tv.up = Pcg{2 * D, 2 * H, 2 * W}.unit(t.n, a.y_up_cstride >> 3, (a.y_up_coffset + ch) >> 3, 2 * t.z, 2 * yy,
+                                                     2 * xx);
+            store_columns(a, tv, ch, lane, vp, r);
+            blk += kConvGroups;
         }
     }
     umma::fence_before_sync();
