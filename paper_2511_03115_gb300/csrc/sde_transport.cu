@@ -597,6 +597,16 @@ __device__ __forceinline__ unsigned long long deposit_chord(const KParams& P, fl
 // deposited total is the sum of the tally, reduced when the balance is read.
 #define SDE_BLOCK_ADD(idx, v) atomicAdd(&s_cnt[idx], (unsigned long long)(v))
 
+// Lanes of a warp that wait with an event until it is sampled for all of them together (or until
+// no other lane can step); each history keeps its own order of operations and random numbers.
+// With the energy-dependent cut-off about one lane in eight has an event per step, so the sampler
+// ran nearly every iteration for the few lanes that had one; waiting lanes miss a step or two
+// instead (3 10^5 protons in the insert phantom, k = 2.5 with secondaries: 2.47 ms without waiting,
+// 2.25 / 2.21 / 2.24 / 2.34 / 2.53 / 3.04 ms for 2 / 3 / 4 / 6 / 8 / 14 lanes).  With the fixed cut-off it
+// is one lane in a hundred, and waiting costs more than it saves (5.61 ms, 5.75 for 2 lanes).
+template <bool CUT>
+constexpr int kEventLanes = CUT ? 3 : 1;
+
 // BR: 0 plain transport; 1 primaries that queue the secondaries of the branching model;
 // 2 the queued secondaries (work items are queue records, not history ids).
 template <int TALLY, bool SMEM, bool AGG, bool CUT, int BR>
@@ -710,7 +720,13 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
         // A large-angle event whose clock fired in the previous step is sampled here,
         // outside the step body, before the history's next step; each history keeps its
         // own order of operations and random numbers.
-        if (jm >= 0) {
+        bool sample = jm >= 0;
+        if (kEventLanes<CUT> > 1) {
+            const unsigned pending = __ballot_sync(0xffffffffu, sample);
+            const unsigned live = __ballot_sync(0xffffffffu, alive);
+            sample = sample && (__popc(pending) >= kEventLanes<CUT> || pending == live);
+        }
+        if (sample) {
             int k;
             float f;
             grid_pos(P, jE, k, f);  // the table position the step's lookup used
@@ -747,7 +763,7 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
                 alive = false;
             }
         }
-        if (!alive) continue;
+        if (!alive || (kEventLanes<CUT> > 1 && jm >= 0)) continue;
 
         if (n >= (uint32_t)P.max_steps || vcur < 0) {  // step cap, or R_n outside the domain D
             if (n >= (uint32_t)P.max_steps) atomicOr(P.err, kErrStepCap);
