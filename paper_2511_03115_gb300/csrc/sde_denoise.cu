@@ -437,11 +437,16 @@ __device__ __forceinline__ void tile_columns(uint32_t tcol, int Cp, float* xch, 
 // channel groups of y (FP32 output: its voxel index), that of its first child on the doubled
 // grid, and whether it is an output voxel.
 struct TileVoxel {
-    size_t at, up;
+    size_t at, up, mask;  // mask: as at, in the mask's tensor
     bool valid;
 };
 
+// What the epilogue does beside bias, leaky ReLU and store: nothing, the upsampled copy, or the
+// adjoint of a leaky ReLU.  Kernels of their own: the code of the others cost the plain one 1 %.
+enum { kConvPlain, kConvUp, kConvMask };
+
 // Bias, leaky ReLU and the stores of the sixteen channels from ch on (tile_columns in r).
+template <int MODE>
 __device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel& t, int ch, int lane, size_t vp,
                                               float2 (&r)[8]) {
     if (a.bias) {
@@ -493,10 +498,22 @@ __device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel
         __nv_bfloat162 pk[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) pk[e] = __float22bfloat162_rn(r[4 * q + e]);
+        if (MODE == kConvMask && t.valid) {  // the value rounded to BF16 first, as a pass of its own would read it
+            const uint4 u = __ldg(reinterpret_cast<const uint4*>(a.mask) + t.mask + q * vp);
+            const __nv_bfloat162* y = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 m = __bfloat1622float2(y[e]);
+                float2 f = __bfloat1622float2(pk[e]);
+                f.x = m.x > 0.f ? f.x : f.x * a.mask_slope;
+                f.y = m.y > 0.f ? f.y : f.y * a.mask_slope;
+                pk[e] = __float22bfloat162_rn(f);
+            }
+        }
         val[q] = *reinterpret_cast<uint4*>(pk);
         if (t.valid) yo[q * vp] = val[q];
     }
-    if (a.y_up) {
+    if (MODE == kConvUp) {
         // The eight children on the doubled grid.  Lane i stores child i & 1 of lane i / 2 (then of lane
         // 16 + i / 2), so that a warp's store covers whole 32-byte sectors: every lane storing its own
         // children left half of each sector to another instruction.
@@ -526,6 +543,7 @@ __device__ __forceinline__ void store_columns(const ConvArgs& a, const TileVoxel
     }
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, BrickPlan b) {
     extern __shared__ __align__(1024) unsigned char smem[];
     // warp-uniform for the compiler too, so that the MMA warps' operands are
@@ -724,10 +742,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
                 tv.at = (size_t)t.n * a.nvox + ((size_t)t.z * H + yy) * W + xx;
             else
                 tv.at = pg.unit(t.n, Gy, (a.y_coffset + ch) >> 3, t.z, yy, xx);
-            if (a.y_up)
+            if (MODE == kConvMask) tv.mask = pg.unit(t.n, a.mask_cstride >> 3, (a.mask_coffset + ch) >> 3, t.z, yy, xx);
+            if (MODE == kConvUp)
                 tv.up = Pcg{2 * D, 2 * H, 2 * W}.unit(t.n, a.y_up_cstride >> 3, (a.y_up_coffset + ch) >> 3, 2 * t.z, 2 * yy,
                                                      2 * xx);
-            store_columns(a, tv, ch, lane, vp, r);
+            store_columns<MODE>(a, tv, ch, lane, vp, r);
             blk += kConvGroups;
         }
     }
@@ -1217,14 +1236,18 @@ cudaError_t conv3d_launch(const ConvArgs& a, int batch, cudaStream_t st) {
     size_t bsmem = 0;
     if (!brick_plan(a.D, a.H, a.W, a.Cin, a.Cout, batch, &bp, &bsmem) || bp.Cp != a.wpk_cp)
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_conv3d_brick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem);
+    auto* kernel = a.y_up   ? k_conv3d_brick<kConvUp>
+                   : a.mask ? k_conv3d_brick<kConvMask>
+                            : k_conv3d_brick<kConvPlain>;
+    if (a.y_up && a.mask) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int ctas = bp.items < sms ? bp.items : sms;
-    k_conv3d_brick<<<ctas, kConvThreads, bsmem, st>>>(a, bp);
+    kernel<<<ctas, kConvThreads, bsmem, st>>>(a, bp);
     return cudaGetLastError();
 }
 
@@ -1401,6 +1424,9 @@ extern "C" int sde_conv3d_forward(const void* d_x, int batch, int D, int H, int 
     a.y_keep = 0;
     a.y_up = nullptr;
     a.y_up_cstride = a.y_up_coffset = 0;
+    a.mask = nullptr;
+    a.mask_cstride = a.mask_coffset = 0;
+    a.mask_slope = 0.f;
     a.relu = relu;
     a.slope = 0.f;
     a.status = d_status;

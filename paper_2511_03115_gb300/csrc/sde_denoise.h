@@ -43,6 +43,12 @@ struct ConvArgs {
     // channel y_up_coffset of y_up_cstride
     void* y_up;
     int y_up_cstride, y_up_coffset;
+    // BF16 output only, optional: the adjoint of a leaky ReLU on the stored values, which are multiplied
+    // by mask_slope where mask (channels mask_coffset .. of mask_cstride, the activation's output) is
+    // not positive
+    const __nv_bfloat16* mask;
+    int mask_cstride, mask_coffset;
+    float mask_slope;
     float slope;  // with relu: y = x > 0 ? x : slope * x (0: ReLU, > 0: leaky ReLU)
     unsigned int* status;
 };

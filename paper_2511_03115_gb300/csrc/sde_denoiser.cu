@@ -134,30 +134,43 @@ __global__ void k_avgpool2(const bf16* __restrict__ in, int ics, int ico, int C,
     st8(out + 8 * coarse_unit(g, c, C >> 3, c.q), acc);
 }
 
-// din (C channels, fine) = dout[parent] / 8 + add (channels aco .. aco+C of acs; may be NULL)
+// The adjoint of the leaky ReLU on a gradient about to be stored: f rounded to BF16, times the
+// slope where the activation's output y (the sign of its pre-activation) is not positive.  The
+// producers of the gradients apply it; as a pass of its own it read and wrote them again (0.45 ms
+// of a 192x128x128 training step).
+__device__ __forceinline__ void relu_bwd8(float (&f)[8], const bf16* y, float slope) {
+    float t[8];
+    ld8(y, t);
+    for (int e = 0; e < 8; ++e) {
+        f[e] = __bfloat162float(__float2bfloat16_rn(f[e]));
+        if (!(t[e] > 0.f)) f[e] *= slope;
+    }
+}
+
+// din (C channels, fine) = dout[parent] / 8 + add (channels aco .. aco+C of acs), through the leaky
+// ReLU whose output is y (channels yco .. of ycs)
 __global__ void k_avgpool2_bwd(const bf16* __restrict__ dout, const bf16* __restrict__ add, int acs, int aco, int C,
-                               Grid2 g, bf16* __restrict__ din) {
+                               Grid2 g, const bf16* __restrict__ y, int ycs, int yco, float slope,
+                               bf16* __restrict__ din) {
     CoarseIdx c;
     if (!coarse_idx(g, C >> 3, c)) return;
     float f[8];
     ld8(dout + 8 * coarse_unit(g, c, C >> 3, c.q), f);
     for (int e = 0; e < 8; ++e) f[e] *= 0.125f;
     for (int d = 0; d < 8; ++d) {
-        float o[8];
-        for (int e = 0; e < 8; ++e) o[e] = f[e];
-        if (add) {
-            float a[8];
-            ld8(add + 8 * fine_unit(g, c, acs >> 3, (aco >> 3) + c.q, d), a);
-            for (int e = 0; e < 8; ++e) o[e] += a[e];
-        }
+        float o[8], a[8];
+        ld8(add + 8 * fine_unit(g, c, acs >> 3, (aco >> 3) + c.q, d), a);
+        for (int e = 0; e < 8; ++e) o[e] = f[e] + a[e];
+        relu_bwd8(o, y + 8 * fine_unit(g, c, ycs >> 3, (yco >> 3) + c.q, d), slope);
         st8(din + 8 * fine_unit(g, c, C >> 3, c.q, d), o);
     }
 }
 
-// dout (C channels, coarse) = sum over the 8 children of din (channels ico .. ico+C of ics):
-// the adjoint of the nearest-neighbour upsampling that the convolution epilogue does
+// dout (C channels, coarse) = sum over the 8 children of din (channels ico .. ico+C of ics), through
+// the leaky ReLU whose output is y (C channels): the adjoint of the nearest-neighbour upsampling
+// that the convolution epilogue does
 __global__ void k_upsample2_bwd(const bf16* __restrict__ din, int ics, int ico, int C, Grid2 g,
-                                bf16* __restrict__ dout) {
+                                const bf16* __restrict__ y, float slope, bf16* __restrict__ dout) {
     CoarseIdx c;
     if (!coarse_idx(g, C >> 3, c)) return;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -166,6 +179,7 @@ __global__ void k_upsample2_bwd(const bf16* __restrict__ din, int ics, int ico, 
         ld8(din + 8 * fine_unit(g, c, ics >> 3, (ico >> 3) + c.q, d), f);
         for (int e = 0; e < 8; ++e) acc[e] += f[e];
     }
+    relu_bwd8(acc, y + 8 * coarse_unit(g, c, C >> 3, c.q), slope);
     st8(dout + 8 * coarse_unit(g, c, C >> 3, c.q), acc);
 }
 
@@ -177,23 +191,6 @@ static bool coarse_grid(const Grid2& g, int C, int batch, dim3& grid) {
     if (z > 65535 || g.C.H > 65535) return false;
     grid = dim3((unsigned)((g.C.W * G + 255) / 256), (unsigned)g.C.H, (unsigned)z);
     return true;
-}
-
-// Leaky ReLU backward over the whole padded tensors (the border is zero in both and stays
-// zero): dy[u] *= (y > 0 ? 1 : slope), y the matching group of channels yco .. of ycs
-// (y has the sign of the pre-activation).  units = batch x C/8 x padded voxels.
-__global__ void k_relu_bwd(bf16* __restrict__ dy, const bf16* __restrict__ y, int ycs, int yco, int C, int units,
-                           int vp, float slope) {
-    const int G = C >> 3;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < units; i += gridDim.x * blockDim.x) {
-        const int r = i / vp, v = i - r * vp, q = r % G, b = r / G;
-        float f[8], t[8];
-        ld8(dy + (size_t)8 * i, f);
-        ld8(y + 8 * (((size_t)b * (ycs >> 3) + (yco >> 3) + q) * vp + v), t);
-        for (int e = 0; e < 8; ++e)
-            if (!(t[e] > 0.f)) f[e] *= slope;
-        st8(dy + (size_t)8 * i, f);
-    }
 }
 
 // db[8q + e] += sum over voxels of channel 8q + e of dy (padded channel-group-major, G = C/8
@@ -531,7 +528,7 @@ struct HostRng {
 // gradient (dy convolved with the flipped weights, Cin and Cout exchanged).
 int conv(sde_denoiser* d, const bf16* x, int batch, int D, int H, int W, const Layer& l, bool flip, int Cout,
          void* y, int cstride, int coffset, bool fp32, bool relu, const float* bias, int keep = 0,
-         bf16* up = nullptr, int up_cstride = 0, int up_coffset = 0) {
+         bf16* up = nullptr, int up_cstride = 0, int up_coffset = 0, const bf16* mask = nullptr) {
     unsigned int* status = nullptr;
     int rc = fail(denoise_status_word(&status), "status word");
     if (rc) return rc;
@@ -554,6 +551,10 @@ int conv(sde_denoiser* d, const bf16* x, int batch, int D, int H, int W, const L
     a.y_up = up;
     a.y_up_cstride = up_cstride;
     a.y_up_coffset = up_coffset;
+    a.mask = mask;  // the activation before the layer, whose gradient this is: all its channels
+    a.mask_cstride = Cout;
+    a.mask_coffset = 0;
+    a.mask_slope = kLeak;
     a.relu = relu ? 1 : 0;
     a.slope = kLeak;
     a.status = status;
@@ -583,12 +584,6 @@ int wgrad(sde_denoiser* d, const bf16* x, const bf16* dy, const Layer& l, int ba
     const dim3 grid((unsigned)(kBlocks / G > 1 ? kBlocks / G : 1), (unsigned)G);
     k_bias_grad<<<grid, 256, 0, d->st>>>(dy, batch, vp, G, l.gb);
     return fail(cudaGetLastError(), "bias grad launch");
-}
-
-int relu_bwd(sde_denoiser* d, bf16* dy, const bf16* y, int ycs, int yco, int C, int batch, const Pcg& g) {
-    const int vp = (int)g.vp();
-    k_relu_bwd<<<kBlocks, 256, 0, d->st>>>(dy, y, ycs, yco, C, batch * (C >> 3) * vp, vp, kLeak);
-    return fail(cudaGetLastError(), "relu bwd launch");
 }
 
 #define DN_TRY(x)              \
@@ -635,50 +630,37 @@ int backward(sde_denoiser* d, int batch) {
     const int D = d->D, H = d->H, W = d->W;
     const int D2 = D / 2, H2 = H / 2, W2 = W / 2, D3 = D / 4, H3 = H / 4, W3 = W / 4;
     const Grid2 g1 = grid2(D, H, W), g2 = grid2(D2, H2, W2);
-    const Pcg& P1 = g1.F;
-    const Pcg& P2 = g2.F;
-    const Pcg& P3 = g2.C;
     Layer* L = d->L;
     dim3 grid;
     // out layer
     DN_TRY(wgrad(d, d->d1, d->g_out, L[10], batch, D, H, W));
-    DN_TRY(conv(d, d->g_out, batch, D, H, W, L[10], true, 32, d->g_d1, 32, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_d1, d->d1, 32, 0, 32, batch, P1));
+    DN_TRY(conv(d, d->g_out, batch, D, H, W, L[10], true, 32, d->g_d1, 32, 0, false, false, nullptr, 0, nullptr, 0, 0, d->d1));
     DN_TRY(wgrad(d, d->d1a, d->g_d1, L[9], batch, D, H, W));
-    DN_TRY(conv(d, d->g_d1, batch, D, H, W, L[9], true, 32, d->g_d1a, 32, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_d1a, d->d1a, 32, 0, 32, batch, P1));
+    DN_TRY(conv(d, d->g_d1, batch, D, H, W, L[9], true, 32, d->g_d1a, 32, 0, false, false, nullptr, 0, nullptr, 0, 0, d->d1a));
     DN_TRY(wgrad(d, d->cat1, d->g_d1a, L[8], batch, D, H, W));
     DN_TRY(conv(d, d->g_d1a, batch, D, H, W, L[8], true, 96, d->g_cat1, 96, 0, false, false, nullptr));
     coarse_grid(g1, 64, batch, grid);
-    k_upsample2_bwd<<<grid, 256, 0, d->st>>>(d->g_cat1, 96, 0, 64, g1, d->g_d2);
-    DN_TRY(relu_bwd(d, d->g_d2, d->d2, 64, 0, 64, batch, P2));
+    k_upsample2_bwd<<<grid, 256, 0, d->st>>>(d->g_cat1, 96, 0, 64, g1, d->d2, kLeak, d->g_d2);
     DN_TRY(wgrad(d, d->d2a, d->g_d2, L[7], batch, D2, H2, W2));
-    DN_TRY(conv(d, d->g_d2, batch, D2, H2, W2, L[7], true, 64, d->g_d2a, 64, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_d2a, d->d2a, 64, 0, 64, batch, P2));
+    DN_TRY(conv(d, d->g_d2, batch, D2, H2, W2, L[7], true, 64, d->g_d2a, 64, 0, false, false, nullptr, 0, nullptr, 0, 0, d->d2a));
     DN_TRY(wgrad(d, d->cat2, d->g_d2a, L[6], batch, D2, H2, W2));
     DN_TRY(conv(d, d->g_d2a, batch, D2, H2, W2, L[6], true, 192, d->g_cat2, 192, 0, false, false, nullptr));
     coarse_grid(g2, 128, batch, grid);
-    k_upsample2_bwd<<<grid, 256, 0, d->st>>>(d->g_cat2, 192, 0, 128, g2, d->g_b2);
-    DN_TRY(relu_bwd(d, d->g_b2, d->b2, 128, 0, 128, batch, P3));
+    k_upsample2_bwd<<<grid, 256, 0, d->st>>>(d->g_cat2, 192, 0, 128, g2, d->b2, kLeak, d->g_b2);
     DN_TRY(wgrad(d, d->b1, d->g_b2, L[5], batch, D3, H3, W3));
-    DN_TRY(conv(d, d->g_b2, batch, D3, H3, W3, L[5], true, 128, d->g_b1, 128, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_b1, d->b1, 128, 0, 128, batch, P3));
+    DN_TRY(conv(d, d->g_b2, batch, D3, H3, W3, L[5], true, 128, d->g_b1, 128, 0, false, false, nullptr, 0, nullptr, 0, 0, d->b1));
     DN_TRY(wgrad(d, d->p2, d->g_b1, L[4], batch, D3, H3, W3));
     DN_TRY(conv(d, d->g_b1, batch, D3, H3, W3, L[4], true, 64, d->g_p2, 64, 0, false, false, nullptr));
     coarse_grid(g2, 64, batch, grid);
-    k_avgpool2_bwd<<<grid, 256, 0, d->st>>>(d->g_p2, d->g_cat2, 192, 128, 64, g2, d->g_e2);
-    DN_TRY(relu_bwd(d, d->g_e2, d->cat2, 192, 128, 64, batch, P2));
+    k_avgpool2_bwd<<<grid, 256, 0, d->st>>>(d->g_p2, d->g_cat2, 192, 128, 64, g2, d->cat2, 192, 128, kLeak, d->g_e2);
     DN_TRY(wgrad(d, d->e2a, d->g_e2, L[3], batch, D2, H2, W2));
-    DN_TRY(conv(d, d->g_e2, batch, D2, H2, W2, L[3], true, 64, d->g_e2a, 64, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_e2a, d->e2a, 64, 0, 64, batch, P2));
+    DN_TRY(conv(d, d->g_e2, batch, D2, H2, W2, L[3], true, 64, d->g_e2a, 64, 0, false, false, nullptr, 0, nullptr, 0, 0, d->e2a));
     DN_TRY(wgrad(d, d->p1, d->g_e2a, L[2], batch, D2, H2, W2));
     DN_TRY(conv(d, d->g_e2a, batch, D2, H2, W2, L[2], true, 32, d->g_p1, 32, 0, false, false, nullptr));
     coarse_grid(g1, 32, batch, grid);
-    k_avgpool2_bwd<<<grid, 256, 0, d->st>>>(d->g_p1, d->g_cat1, 96, 64, 32, g1, d->g_e1);
-    DN_TRY(relu_bwd(d, d->g_e1, d->cat1, 96, 64, 32, batch, P1));
+    k_avgpool2_bwd<<<grid, 256, 0, d->st>>>(d->g_p1, d->g_cat1, 96, 64, 32, g1, d->cat1, 96, 64, kLeak, d->g_e1);
     DN_TRY(wgrad(d, d->e1a, d->g_e1, L[1], batch, D, H, W));
-    DN_TRY(conv(d, d->g_e1, batch, D, H, W, L[1], true, 32, d->g_e1a, 32, 0, false, false, nullptr));
-    DN_TRY(relu_bwd(d, d->g_e1a, d->e1a, 32, 0, 32, batch, P1));
+    DN_TRY(conv(d, d->g_e1, batch, D, H, W, L[1], true, 32, d->g_e1a, 32, 0, false, false, nullptr, 0, nullptr, 0, 0, d->e1a));
     DN_TRY(wgrad(d, d->in0, d->g_e1a, L[0], batch, D, H, W));
     return fail(cudaGetLastError(), "backward launch");
 }
