@@ -132,5 +132,7 @@ cudaError_t wgrad_launch(const WgradArgs& a, cudaStream_t st);
 cudaError_t flip_weights_launch(const __nv_bfloat16* w, __nv_bfloat16* wd, int Cin, int Cout, cudaStream_t st);
 cudaError_t denoise_status_word(unsigned int** out);
 int denoise_check_status(cudaStream_t st);
+// Gives the scratch pool's unused memory on the current device back.
+void denoise_scratch_trim();
 
 }  // namespace sde

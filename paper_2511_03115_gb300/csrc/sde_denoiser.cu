@@ -840,6 +840,7 @@ extern "C" void sde_denoiser_destroy(sde_denoiser* d) {
     cudaStreamSynchronize(d->st);
     free_denoiser(d);
     delete d;
+    denoise_scratch_trim();
 }
 
 extern "C" int sde_denoiser_set_stream(sde_denoiser* d, void* stream) {
