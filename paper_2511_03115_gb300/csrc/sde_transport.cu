@@ -335,13 +335,13 @@ __device__ __forceinline__ bool sde_step_cont(const KParams& P, const float4* ta
     // Lynch-Dahl: w = chi_c^2/(2 chi_alpha^2 (1-F)), sigma^2 = chi_c^2/(1+F^2) g(w),
     // g(w) = (1+w)/w ln(1+w) - 1; Brownian time t = sigma^2 Delta / z.
     float w = rho * ph.w;
-    float g;
-    if (w >= 1.f)
-        g = __fdividef(1.f + w, w) * __logf(1.f + w) - 1.f;
-    else if (w >= 0.01f)
-        g = __fdividef(1.f + w, w) * log1pf(w) - 1.f;
-    else
-        g = w * (0.5f + w * (-1.f / 6.f + w * (1.f / 12.f)));
+    float g = __fdividef(1.f + w, w) * __logf(1.f + w) - 1.f;
+    if (w < 1.f) {  // thin media: the usual case above runs straight through
+        if (w >= 0.01f)
+            g = __fdividef(1.f + w, w) * log1pf(w) - 1.f;
+        else
+            g = w * (0.5f + w * (-1.f / 6.f + w * (1.f / 12.f)));
+    }
     const float t_raw = rho * ph.tg * g;  // sigma^2 Delta / z, whether or not scattering is on
     float t = t_raw * P.mcs_on;
     float th2 = -2.f * t * __logf(u01(x.z));
