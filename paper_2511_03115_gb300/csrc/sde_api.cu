@@ -400,6 +400,7 @@ static KParams make_kparams(const sde_dose* d, int n_spots, uint64_t seed) {
     P.spots = d->d_spots;
     P.prefix = d->d_prefix;
     P.h_end = ~0ull;
+    P.sms = d->num_sms;
     P.n_spots = n_spots;
     P.counters = d->d_counters;
     P.err = d->d_err;
@@ -432,6 +433,7 @@ static int enqueue_branching(sde_dose* d, KParams P, const sde_spot* raw, int n,
         const uint64_t e = std::min<uint64_t>(end, b + kSecQueueCap);
         CUDA_TRY(launch_branch_chunk(d->d_counters, d->d_secctl, b, d->stream));
         P.branch = 1;
+        P.h_begin = b;
         P.h_end = e;
         CUDA_TRY(launch_transport(P, grid, block, 0, false, d->stream));
         P.branch = 2;
@@ -444,6 +446,7 @@ static int enqueue_branching(sde_dose* d, KParams P, const sde_spot* raw, int n,
 static int enqueue_transport(sde_dose* d, const sde_spot* raw, int n, uint64_t seed, uint64_t h_begin = 0,
                              uint64_t h_end = ~0ull) {
     KParams P = make_kparams(d, n, seed);
+    P.h_begin = h_begin;
     P.h_end = h_end;
     int warps = d->tune.warps_per_block;
     int block = warps * 32;

@@ -274,6 +274,7 @@ extern "C" int sde_transport_noalloc(int nx, int ny, int nz, const double voxel_
     P.spots = spots;
     P.prefix = prefix;
     P.h_end = ~0ull;
+    P.sms = sms;
     P.n_spots = n_spots;
     P.counters = counters;
     P.err = err;

@@ -611,8 +611,29 @@ constexpr int kEventLanes = CUT ? 3 : 1;
 // 2 the queued secondaries (work items are queue records, not history ids).
 template <int TALLY, bool SMEM, bool AGG, bool CUT, int BR>
 __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_constant__ KParams P) {
+    unsigned long long total = P.prefix[P.n_spots] < P.h_end ? P.prefix[P.n_spots] : P.h_end;
+    if (BR == 2) total = P.sec_ctl[0] < P.sec_cap ? P.sec_ctl[0] : P.sec_cap;
+    // Small runs are bound by the longest history's chain of steps, and a warp alone on its scheduler
+    // steps fastest.  So blocks past what the histories fill (block b shares a multiprocessor with
+    // b + sms) leave at once; of a block's warps only one per scheduler takes histories while
+    // those last for no more; and they share them evenly, fewer than 32 a warp.  With all resident warps
+    // claiming, the first blocks took everything, eight warps a multiprocessor.  10^4 protons of the
+    // pencil beam 287 -> 248 us with the fetch, 10^5 of a 24-spot plan 774 -> 671 us with the dose.
+    const unsigned long long todo = BR == 2 ? total : total > P.h_begin ? total - P.h_begin : 0ull;
+    // the energy-dependent cut-off samples an event every few steps of a full warp: two lighter warps
+    // a scheduler do better there
+    const unsigned long long warps = (CUT ? 8ull : 4ull) * P.sms;
+    const unsigned lanes = todo < 32ull * warps ? (unsigned)((todo + warps - 1) / warps) : 32u;
+    if ((unsigned long long)(blockIdx.x / P.sms) * P.sms * (blockDim.x >> 5) * lanes >= todo) return;
     extern __shared__ float4 s_tab[];
     __shared__ unsigned long long s_cnt[kCntWords];
+    // lanes that take histories, and how many a warp claims (warp-uniform and rarely read: not kept
+    // in registers)
+    __shared__ unsigned s_lane_mask, s_claim;
+    if (threadIdx.x == 0) {
+        s_lane_mask = 0xffffffffu >> (32u - lanes);
+        s_claim = lanes < 32u ? lanes : (unsigned)P.batch;
+    }
     // The warp's current batch of history ids [next, end) is warp-uniform: it lives in
     // shared memory, not in four registers of every lane.
     __shared__ unsigned long long s_batch[2 * kMaxWarpsPerBlock];
@@ -626,8 +647,6 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    unsigned long long total = P.prefix[P.n_spots] < P.h_end ? P.prefix[P.n_spots] : P.h_end;
-    if (BR == 2) total = P.sec_ctl[0] < P.sec_cap ? P.sec_ctl[0] : P.sec_cap;
     unsigned long long* const cursor = BR == 2 ? &P.sec_ctl[1] : &P.counters[kCntCursor];
     bool alive = false;
     // position (voxel units) and direction; x and y as pairs for packed FP32x2 arithmetic
@@ -648,25 +667,26 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
     uint4 x = make_uint4(0u, 0u, 0u, 0u);
     unsigned long long* const s_next = &s_batch[2 * (threadIdx.x >> 5)];
     unsigned long long* const s_end = s_next + 1;
-    bool drained = false;
+    // warps 4.. of a block take histories only when four a multiprocessor are not enough
+    bool drained = (threadIdx.x >> 7) * 4ull * P.sms * lanes >= todo;
 
     for (;;) {
         unsigned dead = __ballot_sync(0xffffffffu, !alive);
         // refill when the whole warp is idle, or at least refill_min lanes are; once
         // started, until every lane is busy or the queue is drained
         if (dead == 0xffffffffu || (dead && __popc(dead) >= P.refill_min)) {
-            while (dead && !drained) {
+            while ((dead &= s_lane_mask) && !drained) {
                 unsigned long long b_next = *s_next, b_end = *s_end;
                 if (b_next >= b_end) {
                     unsigned long long base = 0;
-                    if (lane == 0) base = atomicAdd(cursor, (unsigned long long)P.batch);
+                    if (lane == 0) base = atomicAdd(cursor, (unsigned long long)s_claim);
                     base = __shfl_sync(0xffffffffu, base, 0);
                     if (base >= total) {
                         drained = true;
                         break;
                     }
                     b_next = base;
-                    b_end = min(base + (unsigned long long)P.batch, total);
+                    b_end = min(base + (unsigned long long)s_claim, total);
                 }
                 int nd = __popc(dead);
                 unsigned long long avail = b_end - b_next;
@@ -715,6 +735,7 @@ __global__ void __launch_bounds__(256, SDE_MIN_BLOCKS) k_transport(const __grid_
                 __syncwarp();
                 dead = __ballot_sync(0xffffffffu, !alive);
             }
+            dead = __ballot_sync(0xffffffffu, !alive);
         }
         if (dead == 0xffffffffu) break;  // queue drained and every lane idle
         // A large-angle event whose clock fired in the previous step is sampled here,
