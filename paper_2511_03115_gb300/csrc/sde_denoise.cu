@@ -257,8 +257,9 @@ namespace {
 // hold no index division, no dispatch and no address that a step could carry: with those a plane
 // took them 500 cycles whatever its MMAs (100 to 500).  The stages are released a plane at a time,
 // which with two of them keeps five of six planes in flight.  192x128x128: 16 -> 32 channels 150 ->
-// 117 us, 32 -> 32 200 -> 165 (the folded epilogue bounds it: 110 without), 96 -> 32 472 -> 336 (operand
-// reads and copies share the shared memory's port), inference 1.89 -> 1.55 ms.
+// 117 us, 32 -> 32 200 -> 165 (145 with the epilogue's 16-column blocks below; the folded epilogue
+// bounds it: 110 without), 96 -> 32 472 -> 336 (operand reads and copies share the shared memory's
+// port), inference 1.89 -> 1.55 ms (1.46 with those blocks).
 // ----------------------------------------------------------------------------
 constexpr int kPipeStages = 2;
 constexpr int kPipeHeader = 1024;  // barriers, tensor-memory slot, abort flag
@@ -1155,11 +1156,6 @@ __global__ void k_flip_weights(const __nv_bfloat16* w, __nv_bfloat16* wd, int Ci
 
 }  // namespace
 
-cudaError_t flip_weights_launch(const __nv_bfloat16* w, __nv_bfloat16* wd, int Cin, int Cout, cudaStream_t st) {
-    k_flip_weights<<<256, 256, 0, st>>>(w, wd, Cin, Cout);
-    return cudaGetLastError();
-}
-
 // Work decomposition of the pipelined brick kernel for one layer shape: output channels
 // split into parts of Cp, weights resident or streamed, rows per item Ty (the last row block
 // may pass H),
@@ -1249,16 +1245,36 @@ static bool brick_plan(int D, int H, int W, int Cin, int Cout, int batch, BrickP
     return found;
 }
 
-// wpk[part][chunk][tap][core-matrix image of the Cp x 16 tile] = w[part Cp + r][tap][16 chunk + k]
+// Element of wpk = [part][chunk][tap][core-matrix image of the Cp x 16 tile] that holds
+// w[co][tap][ci] of a layer of Cin input channels.
+__device__ __forceinline__ size_t packed_at(int co, int tap, int ci, int Cin, int Cp) {
+    const int part = co / Cp, r = co - part * Cp;
+    const size_t tile = (((size_t)part * (Cin >> 4) + (ci >> 4)) * 27 + tap) * Cp * 16;
+    return tile + umma::core_offset(r, ci & 15, 16) / 2;
+}
+
 static __global__ void k_pack_weights(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wpk, int Cin,
                                int Cout, int Cp) {
-    const int n = Cout * 27 * Cin, nchunk = Cin >> 4;
+    const int n = Cout * 27 * Cin;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int ci = i % Cin, tap = (i / Cin) % 27, co = i / (27 * Cin);
-        const int part = co / Cp, r = co - part * Cp, c = ci >> 4, k = ci & 15;
-        const size_t tile = (((size_t)part * nchunk + c) * 27 + tap) * Cp * 16;
-        wpk[tile + umma::core_offset(r, k, 16) / 2] = w[i];
+        wpk[packed_at(co, tap, ci, Cin, Cp)] = w[i];
     }
+}
+
+static __global__ void k_pack_network(const __grid_constant__ PackNet net) {
+    const int l = blockIdx.y, Cin = net.Cin[l], Cout = net.Cout[l], n = Cout * 27 * Cin;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int ci = i % Cin, tap = (i / Cin) % 27, co = i / (27 * Cin);
+        const __nv_bfloat16 v = net.w[l][i];
+        net.fwd[l][packed_at(co, tap, ci, Cin, net.cp[l])] = v;
+        if (net.bwd[l]) net.bwd[l][packed_at(ci, 26 - tap, co, Cout, net.cpf[l])] = v;
+    }
+}
+
+cudaError_t conv_pack_network(const PackNet& net, int layers, cudaStream_t st) {
+    k_pack_network<<<dim3(128, (unsigned)layers), 256, 0, st>>>(net);
+    return cudaGetLastError();
 }
 
 int conv_plan_cp(int D, int H, int W, int Cin, int Cout) {

@@ -127,9 +127,19 @@ int conv_plan_cp(int D, int H, int W, int Cin, int Cout);
 // wpk = w [Cout][27][Cin] in the tensor core's shared-memory image:
 // [Cout/Cp][Cin/16][27][Cp x 16 K-major core matrices].
 cudaError_t conv_pack_weights(const __nv_bfloat16* w, __nv_bfloat16* wpk, int Cin, int Cout, int Cp, cudaStream_t st);
+// The packed images of a whole network's layers in one launch: fwd[i] = w[i] as conv_pack_weights
+// packs it with cp[i] channels per part, and where bwd[i] is not NULL the weights of the data
+// gradient (wd[ci][26 - tap][co] = w[co][tap][ci]) with cpf[i].
+struct PackNet {
+    static constexpr int kMaxLayers = 16;
+    const __nv_bfloat16* w[kMaxLayers];
+    __nv_bfloat16* fwd[kMaxLayers];
+    __nv_bfloat16* bwd[kMaxLayers];
+    int Cin[kMaxLayers], Cout[kMaxLayers], cp[kMaxLayers], cpf[kMaxLayers];
+};
+cudaError_t conv_pack_network(const PackNet& net, int layers, cudaStream_t st);
 cudaError_t conv3d_launch(const ConvArgs& a, int batch, cudaStream_t st);
 cudaError_t wgrad_launch(const WgradArgs& a, cudaStream_t st);
-cudaError_t flip_weights_launch(const __nv_bfloat16* w, __nv_bfloat16* wd, int Cin, int Cout, cudaStream_t st);
 cudaError_t denoise_status_word(unsigned int** out);
 int denoise_check_status(cudaStream_t st);
 // Gives the scratch pool's unused memory on the current device back.
