@@ -317,7 +317,7 @@ __device__ __forceinline__ Lerp lerp_at(float p, int n) {
 }
 
 constexpr int kGammaMaxSteps = 50;
-constexpr int kGammaChunk = 128;  // voxels a block claims at a time
+constexpr int kGammaClaim = 2;  // groups of 32 voxels a warp claims at a time
 struct GammaCtl {
     unsigned long long evaluated, passed, cursor;
     unsigned int maxbits, pad;
@@ -328,24 +328,30 @@ struct GammaCtl {
 // |dr|^2/dta^2 + (De - Dr)^2/(dd Dr)^2 <= 1.  ctl counts the evaluated and the passing voxels.
 //
 // Most voxels are below the threshold or pass at their own position; the search over the ball
-// (9261 positions at 10 steps) runs only for the rest, which are few and clustered.  So blocks
-// claim chunks of 128 voxels from a cursor, test them one per thread, list those that need the
-// search in shared memory, and each warp then searches one voxel with a lane per (y, x)
-// offset of the disk: the lanes walk the z offsets together, interpolate a plane in x and y only
-// when z crosses into the next voxel, skip the offsets between two planes where no lane's dose
-// can come within the tolerance, and stop as soon as a lane passes.  Bound by instruction
-// issue of that walk.  192x128x128, 2 %/0.5 mm, 10 steps: 10.7 ms with one lane per voxel
-// walking the whole ball, 0.42 ms so.
+// (9261 positions at 10 steps) runs only for the rest, which are clustered.  So a warp claims
+// groups of 32 voxels from a cursor, tests them one per lane, and puts those that need the
+// search up as bit masks in shared memory, from which the block's eight warps take one voxel at
+// a time; it claims again when all masks are empty.  A warp searches its voxel with a lane per
+// (y, x) offset of the disk: the lanes walk the z offsets together, upwards from 0 and then below,
+// interpolate a plane in x and y only when z crosses into the next voxel, skip the offsets
+// between two planes where no lane's dose can come within the tolerance, and stop after a half in
+// which a lane passes; the first lanes are spread over the whole disk, so that what passes does so
+// early.  Bound by instruction issue of that walk (0.8 instructions a cycle and scheduler).
+// 192x128x128, 2 %/0.5 mm, 10 steps, call and wait: 10.7 ms with one lane per voxel walking the
+// whole ball; 0.40 ms with a block's warps waiting for each other at every chunk of 128 voxels, the
+// walk always whole and the lanes going outwards row by row; 0.22 ms so (0.26 without the spread
+// lanes; groups taken far apart in the volume: 3 % slower).
 __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, const float* __restrict__ ev, int nx,
                                                int ny, int nz, float hx, float hy, float hz, float dd, float dta,
                                                double threshold, int steps, GammaCtl* ctl) {
     __shared__ float s_q[3][2 * kGammaMaxSteps + 1];                     // offset a st / h per axis
     __shared__ char2 s_yx[(2 * kGammaMaxSteps + 1) * (2 * kGammaMaxSteps + 1)];  // (y, x) offsets in the disk
     __shared__ float4 s_z[8][2 * kGammaMaxSteps + 1];  // per warp: z offset, its fraction f, 1 - f, voxel
-    __shared__ int s_npairs, s_nlist;
-    __shared__ unsigned long long s_claim;
-    __shared__ unsigned char s_list[kGammaChunk];
-    const size_t n = (size_t)nx * ny * nz;
+    __shared__ int s_npairs;
+    // voxels to search: a group's number above the mask of its 32.  A warp's are refilled by that
+    // warp alone, when they are empty; any warp of the block takes from them.
+    __shared__ unsigned long long s_todo[8 * kGammaClaim];
+    const size_t n = (size_t)nx * ny * nz, groups = (n + 31) / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, side = 2 * steps + 1;
     const float st = dta / steps, inv_dta2 = 1.f / (dta * dta);
     const float thr = (float)(threshold * (double)__uint_as_float(ctl->maxbits));
@@ -355,71 +361,105 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
         s_q[1][i] = o / hy;
         s_q[2][i] = o / hz;
     }
-    if (warp == 0) {  // rows of the disk in the order 0, 1, -1, 2, -2 ...: a pass is usually found near 0
-        int at = 0;
-        for (int p0 = 0; p0 < side * side; p0 += 32) {
-            const int p = p0 + lane, r = p / side;
-            const int b = (r & 1) ? (r + 1) / 2 : -(r / 2), c = p - r * side - steps;
+    if (tid == 0) s_npairs = 0;
+    // first a coarse grid over the whole disk: what passes, passes there as a rule
+    const int coarse = max(steps / 3, 1);
+    for (int fine = 0; fine < 2; ++fine) {
+        __syncthreads();
+        for (int p0 = 0; p0 < side * side; p0 += (int)blockDim.x) {
+            const int p = p0 + tid, row = p / side, b = row - steps, c = p - row * side - steps;
             const float oy = b * st, ox = c * st;
-            const bool in = p < side * side && (ox * ox + oy * oy) * inv_dta2 <= 1.f;
+            const bool in = p < side * side && (ox * ox + oy * oy) * inv_dta2 <= 1.f &&
+                            (b % coarse || c % coarse) == (fine != 0);
             const unsigned m = __ballot_sync(0xffffffffu, in);
-            if (in) s_yx[at + __popc(m & ((1u << lane) - 1u))] = make_char2((signed char)b, (signed char)c);
-            at += __popc(m);
+            int at = lane == 0 ? atomicAdd(&s_npairs, __popc(m)) : 0;
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (in) s_yx[at] = make_char2((signed char)b, (signed char)c);
         }
-        if (lane == 0) s_npairs = at;
     }
+    if (tid < 8 * kGammaClaim) s_todo[tid] = 0;
+    __syncthreads();
+    const int npairs = s_npairs;
     unsigned int evals = 0, passes = 0;
+    bool more = true;  // the cursor has not reached the end
+    // this warp's own first
+    unsigned long long* todo = &s_todo[(lane + kGammaClaim * warp) % (8 * kGammaClaim)];
     for (;;) {
-        __syncthreads();  // the list and the claim of the previous round are no longer read
-        if (tid == 0) {
-            s_claim = atomicAdd(&ctl->cursor, (unsigned long long)kGammaChunk);
-            s_nlist = 0;
-        }
-        __syncthreads();
-        const size_t base = (size_t)s_claim;
-        if (base >= n) break;
-        if (tid < kGammaChunk && base + tid < n) {
-            const float r = ref[base + tid];
-            if (r >= thr && r > 0.f) {
-                evals += 1;
-                if (fabsf(ev[base + tid] - r) <= dd * r)
-                    passes += 1;
-                else
-                    s_list[atomicAdd(&s_nlist, 1)] = (unsigned char)tid;
+        __syncwarp();
+        const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(todo);
+        const unsigned has = __ballot_sync(0xffffffffu, lane < 8 * kGammaClaim && (unsigned)seen != 0u);
+        if (!has) {
+            if (!more) break;
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(&ctl->cursor, (unsigned long long)kGammaClaim);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            more = at < groups;
+            if (!more) continue;
+            float r[kGammaClaim], e[kGammaClaim];
+#pragma unroll
+            for (int q = 0; q < kGammaClaim; ++q) {
+                const size_t i = 32 * (at + q) + lane;
+                r[q] = i < n ? ref[i] : 0.f;
             }
-        }
-        __syncthreads();
-        const int nlist = s_nlist, npairs = s_npairs;
-        for (int j = warp; j < nlist; j += 8) {
-            const size_t i = base + s_list[j];
-            const float r = ref[i];
-            const float tol = dd * r, inv_tol2 = 1.f / (tol * tol);
-            const int ix = (int)(i % nx), iy = (int)((i / nx) % ny), iz = (int)(i / ((size_t)nx * ny));
-            __syncwarp();
-            for (int k = lane; k < side; k += 32) {  // the walk along z is the same for every lane
-                const Lerp z = lerp_at(iz + s_q[2][k], nz);
-                s_z[warp][k] = make_float4((k - steps) * st, z.f, 1 - z.f, __int_as_float(z.i0));
+#pragma unroll
+            for (int q = 0; q < kGammaClaim; ++q) e[q] = r[q] >= thr && r[q] > 0.f ? ev[32 * (at + q) + lane] : 0.f;
+#pragma unroll
+            for (int q = 0; q < kGammaClaim; ++q) {
+                const bool eval = r[q] >= thr && r[q] > 0.f;
+                const bool near = fabsf(e[q] - r[q]) <= dd * r[q];
+                evals += eval;
+                passes += eval && near;
+                const unsigned m = __ballot_sync(0xffffffffu, eval && !near);
+                if (lane == q) atomicExch(todo, (at + q) << 32 | m);
             }
-            __syncwarp();
-            const float reach = tol * 1.00001f;  // no rounding of the test below passes beyond this
+            continue;
+        }
+        const int from = __ffs(has) - 1;
+        unsigned long long i = ~0ull;
+        if (lane == from) {
+            const int bit = __ffs((unsigned)seen) - 1;
+            if (atomicCAS(todo, seen, seen & ~(1ull << bit)) == seen) i = (seen >> 32) * 32 + bit;
+        }
+        i = __shfl_sync(0xffffffffu, i, from);
+        if (i == ~0ull) continue;  // another warp took it
+        const float r = ref[i];
+        const float tol = dd * r, inv_tol2 = 1.f / (tol * tol);
+        int ix, iy, iz;
+        if (n >> 32) {
+            ix = (int)(i % nx), iy = (int)((i / nx) % ny), iz = (int)(i / ((size_t)nx * ny));
+        } else {  // 64-bit divisions would be a quarter of a short search
+            const unsigned row = (unsigned)i / (unsigned)nx;
+            ix = (int)((unsigned)i - row * (unsigned)nx);
+            iz = (int)(row / (unsigned)ny);
+            iy = (int)(row - (unsigned)iz * (unsigned)ny);
+        }
+        for (int k = lane; k < side; k += 32) {  // the walk along z is the same for every lane
+            const Lerp z = lerp_at(iz + s_q[2][k], nz);
+            s_z[warp][k] = make_float4((k - steps) * st, z.f, 1 - z.f, __int_as_float(z.i0));
+        }
+        __syncwarp();
+        const float reach = tol * 1.00001f;  // no rounding of the test below passes beyond this
+        bool found = false;
+        for (int p0 = 0; p0 < npairs && !found; p0 += 32) {
+            const bool have = p0 + lane < npairs;
+            const char2 yx = s_yx[have ? p0 + lane : 0];
+            const float oy = yx.x * st, ox = yx.y * st;
+            const Lerp x = lerp_at(ix + s_q[0][yx.y + steps], nx), y = lerp_at(iy + s_q[1][yx.x + steps], ny);
+            const float* f0 = ev + (size_t)y.i0 * nx;
+            const float* f1 = ev + (size_t)y.i1 * nx;
+            auto plane = [&](int z) {
+                const size_t o = (size_t)z * ny * nx;
+                const float c0 = f0[o + x.i0] * (1 - x.f) + f0[o + x.i1] * x.f;
+                const float c1 = f1[o + x.i0] * (1 - x.f) + f1[o + x.i1] * x.f;
+                return c0 * (1 - y.f) + c1 * y.f;
+            };
             bool pass = false;
-            for (int p0 = 0; p0 < npairs; p0 += 32) {
-                const bool have = p0 + lane < npairs;
-                const char2 yx = s_yx[have ? p0 + lane : 0];
-                const float oy = yx.x * st, ox = yx.y * st;
-                const Lerp x = lerp_at(ix + s_q[0][yx.y + steps], nx), y = lerp_at(iy + s_q[1][yx.x + steps], ny);
-                const float* f0 = ev + (size_t)y.i0 * nx;
-                const float* f1 = ev + (size_t)y.i1 * nx;
-                auto plane = [&](int z) {
-                    const size_t o = (size_t)z * ny * nx;
-                    const float c0 = f0[o + x.i0] * (1 - x.f) + f0[o + x.i1] * x.f;
-                    const float c1 = f1[o + x.i0] * (1 - x.f) + f1[o + x.i1] * x.f;
-                    return c0 * (1 - y.f) + c1 * y.f;
-                };
+            for (int half = 0; half < 2 && !found; ++half) {
+                const int k1 = half ? steps : side;
                 int zc = -2;
                 float lo = 0.f, hi = 0.f;
                 bool cell = false;  // some lane's dose between the two planes may come near r
-                for (int k = 0; k < side; ++k) {
+                for (int k = half ? 0 : steps; k < k1; ++k) {
                     const float4 q = s_z[warp][k];
                     const int z0 = __float_as_int(q.w);
                     if (z0 != zc) {
@@ -432,14 +472,12 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
                     if (!cell) continue;
                     const float d2 = (ox * ox + oy * oy + q.x * q.x) * inv_dta2;
                     const float e = lo * q.z + hi * q.y;
-                    pass |= d2 <= 1.f && d2 + (e - r) * (e - r) * inv_tol2 <= 1.f;
+                    pass |= d2 + (e - r) * (e - r) * inv_tol2 <= 1.f;  // not beyond the ball: d2 alone is above 1
                 }
-                if (__any_sync(0xffffffffu, pass && have)) {
-                    passes += lane == 0 ? 1u : 0u;
-                    break;
-                }
+                found = __any_sync(0xffffffffu, pass && have);
             }
         }
+        passes += found && lane == 0 ? 1u : 0u;
     }
     for (int off = 16; off > 0; off >>= 1) {
         evals += __shfl_down_sync(0xffffffffu, evals, off);
