@@ -54,7 +54,7 @@ LANE_OPS_PER_CLK_PER_SM = 128  # 4 schedulers x 32 lanes, one instruction per cl
 # hash of the kernel's source files); otherwise the line reports null.
 TRANSPORT_SOURCES = ("sde_transport.cu", "sde_internal.cuh", "sde_transport.h")
 TRANSPORT_DRAM = {  # workload -> {"src": sha256 prefix, "bytes": per launch, "note": ...}
-    "plan2000": {"src": "2c263b682767634b", "bytes": 1_496_984_320 + 1_409_387_520, "histories": 100_000_000,
+    "plan2000": {"src": "f376f30a82243562", "bytes": 1_480_223_744 + 1_401_346_304, "histories": 100_000_000,
                  "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the first timed launch of "
                          "`bench.py --steps 2 --warmup 1 --no-denoiser --no-cpu-baseline --no-secondary` "
                          "(1 pass; profiles/k_transport_plan2000.md)"},
@@ -63,9 +63,9 @@ TRANSPORT_DRAM = {  # workload -> {"src": sha256 prefix, "bytes": per launch, "n
 # L2 reduction (tally `red.add.u64`) rate of the transport kernel, from ncu on the plan's first
 # 2e6 histories; reported only while the transport sources match the hash it was taken on.
 TRANSPORT_ATOMICS = {
-    "plan2000": {"src": "2c263b682767634b", "l2_red_pct_of_peak": 14.78, "busiest_l2_slice_pct": 16.77,
-                 "red_sectors": 433_046_965, "euler_steps": 525_487_490,
-                 "note": "ncu lts__t_sectors_srcunit_tex_op_red (.sum, .avg/.max pct_of_peak_sustained_elapsed) of "
+    "plan2000": {"src": "f376f30a82243562", "l2_red_pct_of_peak": 16.56, "busiest_l2_slice_pct": None,
+                 "red_sectors": 433_034_795, "euler_steps": 525_487_490,
+                 "note": "ncu lts__t_sectors_srcunit_tex_op_red (.sum, .avg.pct_of_peak_sustained_elapsed) of "
                          "k_transport in `bench.py --histories 2000000 --no-autotune --steps 1 --warmup 1 "
                          "--e2e-steps 0 --no-denoiser --no-cpu-baseline --no-secondary` "
                          "(profiles/k_transport_plan2000.md)"},
@@ -74,10 +74,10 @@ TRANSPORT_ATOMICS = {
 # Instruction issue of the transport kernel (ncu --set full on the plan's first 2e6 histories,
 # same command as the L2 reduction figures); reported only while the sources match its hash.
 TRANSPORT_ISSUE = {
-    "plan2000": {"src": "2c263b682767634b", "issue_active_pct": 79.81, "lanes_per_warp_instruction": 24.86,
-                 "warp_instructions": 7_517_505_206, "euler_steps": 525_487_490,
-                 "pipe_pct": {"alu": 47.96, "fma": 41.16, "fp64": 25.43, "xu_cycles": 40.29, "lsu": 5.87},
-                 "eligible_warps_per_issue": 3.15,
+    "plan2000": {"src": "f376f30a82243562", "issue_active_pct": 78.26, "lanes_per_warp_instruction": 24.79,
+                 "warp_instructions": 6_546_878_349, "euler_steps": 525_487_490,
+                 "pipe_pct": {"alu": 42.67, "fma": 40.62, "fp64": 28.62, "xu_cycles": 45.13, "lsu": 6.62},
+                 "eligible_warps_per_issue": 3.17,
                  "note": "ncu smsp__issue_active (of active cycles), smsp__thread_inst_executed_per_inst_executed, "
                          "smsp__inst_executed.sum, sm__pipe_*_cycles_active, smsp__average_warps_issue_stalled_"
                          "not_selected_per_issue_active of k_transport in `bench.py --histories 2000000 --no-autotune "
