@@ -326,6 +326,9 @@ struct GammaCtl {
 // Local-normalisation gamma: a reference voxel with dose >= threshold max(ref) passes when some
 // evaluated position within the DTA ball (grid step dta/steps, trilinear) has
 // |dr|^2/dta^2 + (De - Dr)^2/(dd Dr)^2 <= 1.  ctl counts the evaluated and the passing voxels.
+// Positions at the ball's edge pass or not by the rounding of |dr|^2, so its operations are
+// written out: the squares of y and z are rounded, the one of x is not, and what lies beyond the
+// edge has a first term above 1.
 //
 // Most voxels are below the threshold or pass at their own position; the search over the ball
 // (9261 positions at 10 steps) runs only for the rest, which are clustered.  So a warp claims
@@ -346,7 +349,7 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
                                                double threshold, int steps, GammaCtl* ctl) {
     __shared__ float s_q[3][2 * kGammaMaxSteps + 1];                     // offset a st / h per axis
     __shared__ char2 s_yx[(2 * kGammaMaxSteps + 1) * (2 * kGammaMaxSteps + 1)];  // (y, x) offsets in the disk
-    __shared__ float4 s_z[8][2 * kGammaMaxSteps + 1];  // per warp: z offset, its fraction f, 1 - f, voxel
+    __shared__ float4 s_z[8][2 * kGammaMaxSteps + 1];  // per warp: z offset squared, its fraction f, 1 - f, voxel
     __shared__ int s_npairs;
     // voxels to search: a group's number above the mask of its 32.  A warp's are refilled by that
     // warp alone, when they are empty; any warp of the block takes from them.
@@ -435,7 +438,8 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
         }
         for (int k = lane; k < side; k += 32) {  // the walk along z is the same for every lane
             const Lerp z = lerp_at(iz + s_q[2][k], nz);
-            s_z[warp][k] = make_float4((k - steps) * st, z.f, 1 - z.f, __int_as_float(z.i0));
+            const float oz = (k - steps) * st;
+            s_z[warp][k] = make_float4(__fmul_rn(oz, oz), z.f, 1 - z.f, __int_as_float(z.i0));
         }
         __syncwarp();
         const float reach = tol * 1.00001f;  // no rounding of the test below passes beyond this
@@ -443,7 +447,7 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
         for (int p0 = 0; p0 < npairs && !found; p0 += 32) {
             const bool have = p0 + lane < npairs;
             const char2 yx = s_yx[have ? p0 + lane : 0];
-            const float oy = yx.x * st, ox = yx.y * st;
+            const float oy = yx.x * st, ox = yx.y * st, oxy2 = fmaf(ox, ox, __fmul_rn(oy, oy));
             const Lerp x = lerp_at(ix + s_q[0][yx.y + steps], nx), y = lerp_at(iy + s_q[1][yx.x + steps], ny);
             const float* f0 = ev + (size_t)y.i0 * nx;
             const float* f1 = ev + (size_t)y.i1 * nx;
@@ -470,9 +474,9 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
                         cell = __any_sync(0xffffffffu, !(fmaxf(lo, hi) < r - slack) && !(fminf(lo, hi) > r + slack));
                     }
                     if (!cell) continue;
-                    const float d2 = (ox * ox + oy * oy + q.x * q.x) * inv_dta2;
+                    const float d2 = __fmul_rn(__fadd_rn(oxy2, q.x), inv_dta2);
                     const float e = lo * q.z + hi * q.y;
-                    pass |= d2 + (e - r) * (e - r) * inv_tol2 <= 1.f;  // not beyond the ball: d2 alone is above 1
+                    pass |= fmaf((e - r) * (e - r), inv_tol2, d2) <= 1.f;
                 }
                 found = __any_sync(0xffffffffu, pass && have);
             }
