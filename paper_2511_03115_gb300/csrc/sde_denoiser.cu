@@ -327,8 +327,8 @@ struct GammaCtl {
 // evaluated position within the DTA ball (grid step dta/steps, trilinear) has
 // |dr|^2/dta^2 + (De - Dr)^2/(dd Dr)^2 <= 1.  ctl counts the evaluated and the passing voxels.
 // Positions at the ball's edge pass or not by the rounding of |dr|^2, so its operations are
-// written out: the squares of y and z are rounded, the one of x is not, and what lies beyond the
-// edge has a first term above 1.
+// written out, in the search and in the list of the disk's offsets alike: the squares of y and z
+// are rounded, the one of x is not, and what lies beyond the edge has a first term above 1.
 //
 // Most voxels are below the threshold or pass at their own position; the search over the ball
 // (9261 positions at 10 steps) runs only for the rest, which are clustered.  So a warp claims
@@ -342,7 +342,7 @@ struct GammaCtl {
 // early.  Bound by instruction issue of that walk (0.8 instructions a cycle and scheduler).
 // 192x128x128, 2 %/0.5 mm, 10 steps, call and wait: 10.7 ms with one lane per voxel walking the
 // whole ball; 0.40 ms with a block's warps waiting for each other at every chunk of 128 voxels, the
-// walk always whole and the lanes going outwards row by row; 0.22 ms so (0.26 without the spread
+// walk always whole and the lanes going outwards row by row; 0.23 ms so (0.26 without the spread
 // lanes; groups taken far apart in the volume: 3 % slower).
 __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, const float* __restrict__ ev, int nx,
                                                int ny, int nz, float hx, float hy, float hz, float dd, float dta,
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(256) k_gamma(const float* __restrict__ ref, co
         for (int p0 = 0; p0 < side * side; p0 += (int)blockDim.x) {
             const int p = p0 + tid, row = p / side, b = row - steps, c = p - row * side - steps;
             const float oy = b * st, ox = c * st;
-            const bool in = p < side * side && (ox * ox + oy * oy) * inv_dta2 <= 1.f &&
+            const bool in = p < side * side && __fmul_rn(fmaf(ox, ox, __fmul_rn(oy, oy)), inv_dta2) <= 1.f &&
                             (b % coarse || c % coarse) == (fine != 0);
             const unsigned m = __ballot_sync(0xffffffffu, in);
             int at = lane == 0 ? atomicAdd(&s_npairs, __popc(m)) : 0;
