@@ -313,14 +313,14 @@ int sde_conv3d_flip_weights(const void* d_w, void* d_wd, int Cin, int Cout, void
 /* Host-only inspection of the work decompositions of the two convolution kernels
  * (no CUDA call: usable without a GPU, e.g. to check a shape's shared-memory and
  * tensor-memory layout before running it).
- * sde_conv3d_plan: the plan of sde_conv3d_forward for this shape, as 17 ints in the
+ * sde_conv3d_plan: the plan of sde_conv3d_forward for this shape, as 18 ints in the
  * order Ty, tiles, rowtile, fold, nyb, P, Yb, Cp, nsplit, plane, w_off, wres, stage,
- * nacc, xch, tcols, items (rows per work item, 128-position M tiles per item, row
+ * nacc, xch, tcols, items, groups (rows per work item, 128-position M tiles per item, row
  * tiles, x-tap fold, row blocks, brick row pitch W + 2, brick rows Ty + 2, output
  * channels per part, parts, bytes between the two 8-channel planes of a chunk,
  * weight offset in a stage, resident weights, bytes per stage, accumulators,
- * offset of the fold's exchange buffer, tensor-memory columns, work items), and
- * its dynamic shared memory in bytes.
+ * offset of the fold's exchange buffer, tensor-memory columns, work items, epilogue
+ * groups that take part), and its dynamic shared memory in bytes.
  * sde_conv3d_wgrad_plan: the row-block plan of sde_conv3d_wgrad on a GPU with `sms`
  * multiprocessors, as 14 ints: Ty, nyb, P, Yb, Nc, ntap, ngroups, kst, plane_dy,
  * plane_x, x_off, stage, items, G (input channels and taps per pass, tap groups,

@@ -432,7 +432,7 @@ def conv3d(x, w, bias=None, relu=False, y=None, y_coffset=0, fp32=False, stream=
 
 
 CONV_PLAN_FIELDS = ("Ty", "tiles", "rowtile", "fold", "nyb", "P", "Yb", "Cp", "nsplit", "plane", "w_off", "wres",
-                    "stage", "nacc", "xch", "tcols", "items")
+                    "stage", "nacc", "xch", "tcols", "items", "groups")
 WGRAD_PLAN_FIELDS = ("Ty", "nyb", "P", "Yb", "Nc", "ntap", "ngroups", "kst", "plane_dy", "plane_x", "x_off", "stage",
                      "items", "G")
 WGRAD_RING_FIELDS = ("order", "Ty", "gpp", "ngr", "ns", "nt", "kst", "P", "ra", "drun", "dyx", "xoff", "dslot", "xslot",

@@ -724,7 +724,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
     } else {
         // epilogue: the blocks of sixteen columns of the CTA's M tiles, all items' in order, go round
         // the groups.  Each warp waits for its tile's accumulator by itself; after a timeout it goes on
-        // through its blocks without storing, so that the group's barriers still meet.
+        // through its blocks without storing, so that the group's barriers still meet.  A group does not
+        // wait for an item that it has no block of, and a wait tells an accumulator's fillings apart
+        // by their parity only: with one block an item and four groups, the next item of a group is its
+        // accumulator's next but one, whose wait would end at once.  So only as many groups take part as
+        // have a block of every nacc-th item (b.groups).
         const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. + 31
         const int grp = warp >> 2, blocks = Cp >> 4;
         const size_t vp = pg.vp();
@@ -738,7 +742,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
         bool ok = true;
         uint32_t acc_par = 0;
         int acc = 0, m = 0, blk = grp;
-        while (t.left > 0) {
+        while (grp < b.groups && t.left > 0) {
             if (blk >= blocks) {  // on to the next tile
                 blk -= blocks;
                 if (++m < b.tiles) continue;
@@ -791,7 +795,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
                 tv.up = Pcg{2 * D, 2 * H, 2 * W}.unit(t.n, a.y_up_cstride >> 3, (a.y_up_coffset + ch) >> 3, 2 * t.z, 2 * yy,
                                                      2 * xx);
             store_columns<MODE>(a, tv, ch, lane, vp, r);
-            blk += kConvGroups;
+            blk += b.groups;
         }
     }
     umma::fence_before_sync();
@@ -1237,6 +1241,8 @@ static bool brick_plan(int D, int H, int W, int Cin, int Cout, int batch, BrickP
                         bp.xch = (int)xch;
                         bp.tcols = tcols;
                         bp.items = batch * nsplit * nyb * D;
+                        const int turns = nacc * tiles * (Cp / 16);
+                        bp.groups = turns < kConvGroups ? turns : kConvGroups;
                         *out = bp;
                         *smem_out = smem;
                     }
@@ -1542,9 +1548,9 @@ extern "C" int sde_conv3d_plan(int batch, int D, int H, int W, int Cin, int Cout
         set_last_error("sde_conv3d_plan: shape rejected by the convolution or without a plan");
         return SDE_EINVAL;
     }
-    const int32_t v[17] = {bp.Ty,    bp.tiles, bp.rowtile, bp.fold,  bp.nyb, bp.P,    bp.Yb,  bp.Cp,   bp.nsplit,
-                           bp.plane, bp.w_off, bp.wres,    bp.stage, bp.nacc, bp.xch, bp.tcols, bp.items};
-    for (int i = 0; i < n_fields && i < 17; ++i) fields[i] = v[i];
+    const int32_t v[18] = {bp.Ty,    bp.tiles, bp.rowtile, bp.fold,  bp.nyb, bp.P,    bp.Yb,  bp.Cp,   bp.nsplit,
+                           bp.plane, bp.w_off, bp.wres,    bp.stage, bp.nacc, bp.xch, bp.tcols, bp.items, bp.groups};
+    for (int i = 0; i < n_fields && i < 18; ++i) fields[i] = v[i];
     if (smem_bytes) *smem_bytes = smem;
     return SDE_OK;
 }

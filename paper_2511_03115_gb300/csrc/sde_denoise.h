@@ -73,6 +73,7 @@ struct BrickPlan {
     int xch;      // fold: offset of the epilogue's boundary-exchange buffer in shared memory
     int tcols;    // tensor-memory columns allocated (power of two >= nacc x tiles x Cp x (fold ? 3 : 1))
     int items;    // batch x nsplit x nyb x D
+    int groups;   // epilogue groups that take part: at most nacc x tiles x Cp/16
 };
 
 // Weight gradient of the convolution; x and dy padded channel-group-major.
