@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "sde_dose.h"
@@ -833,7 +834,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 // warp at some seven cycles an instruction, so they keep positions, slots and phases by
 // increments: with the index divisions in their loops (three to four thousand cycles an item)
 // they, not the MMAs, set the time.  An item's commits release its dy slot and the planes no later
-// item needs.  dW stays in tensor memory over all of the CTA's items and is added to global memory
+// item needs.  A copying warp waits for a slot by the parity of its fillings, so no filling may go
+// by without it: in the long order only warps that copy a part of every item take part (without it
+// the item's MMAs cannot run), in the short order, where the planes' copies go round the warps, each of
+// them arrives for every filling.  dW stays in tensor memory over all of the CTA's items and is added to global memory
 // at the end, each CTA starting at another column (all walking the same order would meet on the
 // same addresses).
 //
@@ -938,11 +942,11 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
     }
     if (tid == 0) {
         for (int i = 0; i < b.XS; ++i) {
-            umma::mbar_init(&fullx[i], 1);
+            umma::mbar_init(&fullx[i], (uint32_t)b.arrivals);
             umma::mbar_init(&emptyx[i], b.nt);  // one commit per issuer
         }
         for (int i = 0; i < b.DS; ++i) {
-            umma::mbar_init(&fulld[i], 1);
+            umma::mbar_init(&fulld[i], (uint32_t)b.arrivals);
             umma::mbar_init(&emptyd[i], b.nt);
         }
         umma::mbar_init(dfull, b.nt);
@@ -957,7 +961,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
     const bool any = it.left > 0;
 
     if (warp < kRingCopyWarps) {
-        if (lane == 0) {
+        if (lane == 0 && warp < b.copiers) {
             const Pcg pg{D, H, W};
             const int gd = Cout >> 3, nd = b.ns * gd, gx = Cin >> 3;
             const uint32_t xrun = (uint32_t)(Yb * b.P * 16);
@@ -1007,7 +1011,10 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                 for (; it.left > 0; ++j) {
                     if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
                     const size_t at = (size_t)it.z * plane + (size_t)it.yb * (b.P * 16);
-                    if (warp == 0) umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
+                    if (warp == 0)
+                        umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
+                    else
+                        umma::mbar_arrive(&fulld[sd.i]);
 #pragma unroll
                     for (int e = 0; e < 2; ++e)
                         if (mine[e])
@@ -1016,7 +1023,10 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                     const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
                     for (int f = 0; f < fresh; ++f, ++planes) {
                         if (planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag))) break;
-                        if (warp == 0) umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
+                        if (warp == 0)
+                            umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
+                        else
+                            umma::mbar_arrive(&fullx[sx.i]);
                         for (int q = 0; q < b.gpp; ++q, ++turn)
                             if (turn % kRingCopyWarps == warp)
                                 umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
@@ -1417,6 +1427,9 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
                 w.smem = w.x_off + w.XS * w.xslot + (w.P + 32) * 16;
                 if (w.smem < tail) w.smem = tail;
                 if (w.smem <= 227 * 1024) {
+                    const int nd = w.ns * (a.Cout / 8);
+                    w.copiers = order ? std::min(kRingCopyWarps, std::max(nd, 3 * w.gpp)) : kRingCopyWarps;
+                    w.arrivals = order ? 1 : w.copiers;
                     *out = w;
                     return true;
                 }
@@ -1597,9 +1610,9 @@ extern "C" int sde_conv3d_wgrad_ring(int batch, int D, int H, int W, int Cin, in
         set_last_error("sde_conv3d_wgrad_ring: shape rejected by the weight gradient or without a plan");
         return SDE_EINVAL;
     }
-    const int32_t v[19] = {w.order, w.Ty, w.gpp, w.ngr, w.ns,  w.nt,  w.kst,  w.P,     w.ra, w.drun,
-                           w.dyx,   w.xoff, w.dslot, w.xslot, w.DS, w.XS, w.x_off, w.items, w.G};
-    for (int i = 0; i < n_fields && i < 19; ++i) fields[i] = v[i];
+    const int32_t v[21] = {w.order, w.Ty,    w.gpp,   w.ngr, w.ns, w.nt,    w.kst,   w.P, w.ra,      w.drun,    w.dyx,
+                           w.xoff,  w.dslot, w.xslot, w.DS,  w.XS, w.x_off, w.items, w.G, w.copiers, w.arrivals};
+    for (int i = 0; i < n_fields && i < 21; ++i) fields[i] = v[i];
     if (smem_bytes) *smem_bytes = (uint64_t)w.smem;
     return SDE_OK;
 }

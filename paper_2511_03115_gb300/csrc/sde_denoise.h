@@ -120,6 +120,8 @@ struct WgradRing {
     int smem;          // dynamic shared memory in bytes
     int items;         // batch x nyb x D
     int G;             // CTAs per pass
+    int copiers;       // copying warps that take part
+    int arrivals;      // arrivals per filling of a slot: 1 (every copier has a part of each), or all copiers
 };
 
 // Output channels per part that conv3d_launch will use for this layer shape (the packing
