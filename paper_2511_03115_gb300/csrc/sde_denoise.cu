@@ -1381,10 +1381,7 @@ constexpr double kLongSum = 1024.0;
 
 bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing* out) {
     const double steps = (double)wp.items / wp.G * wp.kst;
-    // the last choice, eight channels a pass in the short order, is for rows so wide that two groups
-    // of input rows do not fit beside two dy slots of 128 channels
-    for (int choice = steps > kLongSum && wp.Ty <= 6 ? 0 : 1; choice < 3; ++choice) {
-        const int order = choice == 0 ? 1 : 0;
+    for (int order = steps > kLongSum && wp.Ty <= 6 ? 1 : 0; order >= 0; --order) {
         WgradRing w{};
         w.order = order;
         w.P = a.W + 2;
@@ -1399,7 +1396,10 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
         } else {
             w.Ty = 1;
             w.ns = a.Cout <= 40 ? 3 : a.Cout <= 64 ? 2 : 1;
-            w.gpp = choice == 1 ? 2 : 1;
+            // always two groups of channels: where the ring wraps inside a window the MMA is cut into runs
+            // of gpp Yb row groups, and with one group these would be 24 and 56 columns, which an
+            // MMA of M = 128 does not take (multiples of 16)
+            w.gpp = 2;
             w.kst = (a.W + 15) / 16;
             w.drun = a.W * 16;
             w.dyx = w.ns == 3 ? 1 : 0;  // copy 0 is shifted by s = -1 or 0
@@ -1421,10 +1421,12 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
         for (w.DS = kRingMaxD; w.DS >= 2; --w.DS)
             for (w.XS = order ? 3 * w.DS : kRingMaxX; w.XS >= (order ? 3 * w.DS : w.DS + 2); --w.XS) {
                 w.x_off = kPipeHeader + w.DS * w.dslot;
-                // the windows of the last slot end up to a row and a K step past it, and M = 128 rows of
-                // A start in the last dy slot
+                // the windows of the last three slots may end past them (with rows of 256 and 64 or 128
+                // output channels a more generous end leaves no room for four planes), and M = 128 rows
+                // of A start in the last dy slot
+                const int past = (w.ngr - 1) * w.P + w.xoff + w.nt - 1 + 16 * w.kst - 3 * w.xslot / 16;
                 const int tail = kPipeHeader + (w.DS - 1) * w.dslot + 16 * w.ra;
-                w.smem = w.x_off + w.XS * w.xslot + (w.P + 32) * 16;
+                w.smem = w.x_off + w.XS * w.xslot + (past > 0 ? past : 0) * 16;
                 if (w.smem < tail) w.smem = tail;
                 if (w.smem <= 227 * 1024) {
                     const int nd = w.ns * (a.Cout / 8);
