@@ -327,15 +327,16 @@ int sde_conv3d_flip_weights(const void* d_w, void* d_wd, int Cin, int Cout, void
  * 16-position K steps per item, plane pitches of the output-gradient rows and of
  * the input brick, brick offset in a stage, CTAs per pass), and its dynamic shared
  * memory.  The weight gradient accepts the shapes that have such a plan.
- * sde_conv3d_wgrad_ring: what it launches for them, as 21 ints: order, Ty, gpp, ngr, ns,
+ * sde_conv3d_wgrad_ring: what it launches for them, as 23 ints: order, Ty, gpp, ngr, ns,
  * nt, kst, P, ra, drun, dyx, xoff, dslot, xslot, DS, XS, x_off, items, G, copiers,
- * arrivals (order of the items: 0 contiguous rows, 1 the row-block plan's; rows per item, 8-channel groups
- * per pass, row groups in N, shifted copies of the output-gradient rows in M, offsets
+ * arrivals, load, back (order of the items: 0 contiguous rows, 1 the row-block plan's;
+ * rows per item, 8-channel groups in a plane slot, row groups in N, shifted copies of the output-gradient rows in M, offsets
  * of the x window, 16-position K steps per item, W + 2, bytes of an 8-channel run and
  * of what is copied into it, x of its first position, the x window's first
  * position, bytes of an output-gradient slot and of a plane slot, slots of each,
  * offset of the first plane slot, items, CTAs per pass, copying warps that take part,
- * arrivals per filling of a slot), and its dynamic shared memory.
+ * arrivals per filling of a slot, 8-channel groups loaded per pass, positions that the last
+ * K step's x window starts early), and its dynamic shared memory.
  * All fill min(n_fields, count) ints; SDE_EINVAL for a shape the convolution rejects or
  * has no plan for. */
 int sde_conv3d_plan(int batch, int D, int H, int W, int Cin, int Cout, int32_t* fields, int n_fields,

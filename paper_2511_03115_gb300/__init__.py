@@ -436,7 +436,7 @@ CONV_PLAN_FIELDS = ("Ty", "tiles", "rowtile", "fold", "nyb", "P", "Yb", "Cp", "n
 WGRAD_PLAN_FIELDS = ("Ty", "nyb", "P", "Yb", "Nc", "ntap", "ngroups", "kst", "plane_dy", "plane_x", "x_off", "stage",
                      "items", "G")
 WGRAD_RING_FIELDS = ("order", "Ty", "gpp", "ngr", "ns", "nt", "kst", "P", "ra", "drun", "dyx", "xoff", "dslot", "xslot",
-                     "DS", "XS", "x_off", "items", "G", "copiers", "arrivals")
+                     "DS", "XS", "x_off", "items", "G", "copiers", "arrivals", "load", "back")
 
 
 def conv3d_plan(batch, D, H, W, Cin, Cout):

@@ -823,11 +823,16 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 // results may move by):
 //  - short sums: a CTA owns a contiguous range of rows (Ty = 1) with z running fastest, so each
 //    further row needs one new plane; M is filled with shifted copies (ns = 3 up to 40 channels,
-//    2 up to 64), i.e. 96 of its 128 rows at 32 channels.  Positions past W up to the K step's end
-//    meet zeros in dy (its slots are zeroed once and only W positions are ever written);
+//    2 up to 64), i.e. 96 of its 128 rows at 32 channels;
 //  - long sums: the items, K steps and CTAs of the row-block plan in their order, so that every
 //    sum is formed from the same products in the same order as with one MMA per tap (bit for bit
 //    up to the order of the CTAs' atomics); three offsets t, no copies.
+//
+// A window of x that passed its row's end would bring other channels' values under the zeros that
+// fill dy's last K step, and zero times infinity is no zero.  So the last step's positions lie at its
+// end, behind the zeros, and its window starts that much earlier, over positions that are paired
+// with zeros there.  A row shorter than a K step has no earlier positions: its passes load one
+// group of channels, and the second group's part of each slot stays zero.
 //
 // One thread in each of warps 0-7 brings operands, its share of an item's 10 to 20 bulk copies; one
 // in each of warps 8-10 issues the MMAs of one offset t.  Each of these threads runs alone in its
@@ -851,20 +856,21 @@ constexpr int kRingMaxX = 12, kRingMaxD = 4, kRingCopyWarps = 8, kRingWarps = kR
 // The MMAs of one item, offset and run of planes, issued by a whole warp's leader.  Unrolled,
 // because address arithmetic between two MMAs of one warp costs more than the MMA.
 __device__ __forceinline__ void ring_mma(uint32_t leader, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                         uint32_t b_hi, uint32_t idesc, int kst, uint32_t first) {
+                                         uint32_t b_hi, uint32_t idesc, int kst, int back, uint32_t first) {
     umma::mma_bf16_warp(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, first);
     int ks = 1;
     for (; ks + 4 <= kst; ks += 4) {
+        const uint32_t last = ks + 4 == kst ? (uint32_t)back : 0u;
 #pragma unroll
         for (int u = 1; u <= 4; ++u)
-            umma::mma_bf16_warp(leader, d, a_lo + 16 * u, a_hi, b_lo + 16 * u, b_hi, idesc, 1u);
+            umma::mma_bf16_warp(leader, d, a_lo + 16 * u, a_hi, b_lo + 16 * u - (u == 4 ? last : 0u), b_hi, idesc, 1u);
         a_lo += 64;
         b_lo += 64;
     }
     for (; ks < kst; ++ks) {
         a_lo += 16;
         b_lo += 16;
-        umma::mma_bf16_warp(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, 1u);
+        umma::mma_bf16_warp(leader, d, a_lo, a_hi, b_lo - (ks + 1 == kst ? (uint32_t)back : 0u), b_hi, idesc, 1u);
     }
 }
 
@@ -930,7 +936,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
     uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 320);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 324);
     const uint32_t s_d = umma::smem_addr(smem) + kPipeHeader, s_x = umma::smem_addr(smem) + (uint32_t)b.x_off;
-    const int c = blockIdx.y;  // chunk of 8 gpp input channels
+    const int c = blockIdx.y;  // chunk of 8 load input channels
     {  // what the copies never write must read as zero, not leftover bits (0 x NaN is NaN)
         uint4* z = reinterpret_cast<uint4*>(smem + kPipeHeader);
         for (int i = tid; i < (b.smem - kPipeHeader) / 16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -965,6 +971,13 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
             const Pcg pg{D, H, W};
             const int gd = Cout >> 3, nd = b.ns * gd, gx = Cin >> 3;
             const uint32_t xrun = (uint32_t)(Yb * b.P * 16);
+            // a dy run's copies: its whole K steps, and the last one's positions at that step's end
+            const uint32_t dmain = (uint32_t)(b.back ? (b.kst - 1) * 256 : b.drun), dtail = (uint32_t)b.drun - dmain;
+            const uint32_t tail_at = dmain + 16u * (uint32_t)b.back;
+            auto copy_dy = [&](uint32_t dst, const unsigned char* src, uint64_t* full) {
+                umma::bulk_g2s(dst, src, dmain, full);
+                if (dtail) umma::bulk_g2s(dst + tail_at, src + dmain, dtail, full);
+            };
             const size_t plane = (size_t)(H + 2) * b.P * 16, vp = pg.vp() * 16;
             // this warp's dy copies (copy i / gd of channel group i % gd; at most 16 in all) and the
             // plane copies' sources, at z = y0 = n = 0
@@ -978,7 +991,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                 ddst[e] = s_d + (uint32_t)(i * b.ra);
             }
             const unsigned char* xsrc =
-                reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.gpp, -1, -1, -1));
+                reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.load, -1, -1, -1));
             RingSlot sd;
             int j = 0;
             bool ok = true;
@@ -999,8 +1012,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
 #pragma unroll
                     for (int e = 0; e < 2; ++e)
                         if (mine[e])
-                            umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
-                                           (uint32_t)b.drun, full);
+                            copy_dy(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp, full);
                     sd.advance(b.DS);
                     it.next(b, D);
                 }
@@ -1018,16 +1030,16 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
 #pragma unroll
                     for (int e = 0; e < 2; ++e)
                         if (mine[e])
-                            umma::bulk_g2s(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
-                                           (uint32_t)b.drun, &fulld[sd.i]);
+                            copy_dy(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
+                                    &fulld[sd.i]);
                     const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
                     for (int f = 0; f < fresh; ++f, ++planes) {
                         if (planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag))) break;
                         if (warp == 0)
-                            umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.gpp * xrun);
+                            umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.load * xrun);
                         else
                             umma::mbar_arrive(&fullx[sx.i]);
-                        for (int q = 0; q < b.gpp; ++q, ++turn)
+                        for (int q = 0; q < b.load; ++q, ++turn)
                             if (turn % kRingCopyWarps == warp)
                                 umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
                                                &fullx[sx.i]);
@@ -1062,7 +1074,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                 ok = pipe_wait(&fulld[sd.i], sd.par, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) break;
                 umma::fence_after_sync();
-                ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, accum);
+                ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, b.back, accum);
                 accum = 1;
                 umma::mma_commit_warp(leader, &emptyd[sd.i]);
                 sd.advance(b.DS);
@@ -1084,12 +1096,12 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                 const uint32_t b_lo = (uint32_t)b0 + (uint32_t)k * xstep;
                 const int run = b.XS - k;  // planes before the ring wraps
                 if (run >= 3) {
-                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, accum);
+                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, b.back, accum);
                 } else {
                     const int n1 = run * gp;
-                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, accum);
+                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, b.back, accum);
                     ring_mma(leader, d + (uint32_t)(8 * n1), a_lo, a_hi, (uint32_t)b0, b_hi,
-                             umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, accum);
+                             umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, b.back, accum);
                 }
                 accum = 1;
                 umma::mma_commit_warp(leader, &emptyd[sd.i]);
@@ -1133,13 +1145,13 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                     const int t = cell / b.ngr, q = cell - t * b.ngr;
                     const int r = q % Yb, pg = q / Yb, dz = pg / b.gpp, g = pg - dz * b.gpp;
                     const int dx = t + i - 1;
-                    if (r > 2 || dz > 2) continue;  // rows between the taps
+                    if (r > 2 || dz > 2 || g >= b.load) continue;  // rows between the taps, groups not loaded
                     float v[8];
                     __syncwarp();
                     umma::tmem_ld8(tbase + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(t * N + 8 * q), v);
                     // two copies give dx = 0 twice, the second time (s = 1, t = -1) without the last position
                     if (i < b.ns && !(b.ns == 2 && i == 1 && t == 0)) {
-                        float* d = a.dw + ((size_t)co * 27 + 9 * dz + 3 * r + dx + 1) * Cin + 8 * (c * b.gpp + g);
+                        float* d = a.dw + ((size_t)co * 27 + 9 * dz + 3 * r + dx + 1) * Cin + 8 * (c * b.load + g);
                         if (vec) {
                             atomicAdd(reinterpret_cast<float4*>(d), make_float4(v[0], v[1], v[2], v[3]));
                             atomicAdd(reinterpret_cast<float4*>(d) + 1, make_float4(v[4], v[5], v[6], v[7]));
@@ -1388,7 +1400,8 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
         if (order) {
             w.Ty = wp.Ty;
             w.ns = 1;
-            w.gpp = wp.Ty == 1 ? 2 : 1;  // what three accumulators in tensor memory leave room for
+            // what three accumulators in tensor memory leave room for; one where a K step passes the rows
+            w.gpp = wp.Ty == 1 && wp.kst > 1 ? 2 : 1;
             w.kst = wp.kst;
             w.drun = w.Ty * w.P * 16;  // rows with their padding, from x = -1
             w.dyx = -1;
@@ -1404,12 +1417,15 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
             w.drun = a.W * 16;
             w.dyx = w.ns == 3 ? 1 : 0;  // copy 0 is shifted by s = -1 or 0
         }
+        const int used = w.drun / 16 - 16 * (w.kst - 1);  // positions of the last K step
+        w.back = w.kst > 1 ? 16 - used : 0;
+        w.load = w.kst > 1 || used == 16 ? w.gpp : 1;
         w.nt = w.ns == 3 ? 1 : w.ns == 2 ? 2 : 3;
         // the window of t = t0 at the first position: the slot's rows start at x = -1
         w.xoff = order ? -1 : w.nt == 1 ? 1 : 0;
         w.nyb = a.H / w.Ty;
         w.items = a.batch * w.nyb * a.D;
-        const int Yb = w.Ty + 2, passes = a.Cin / (8 * w.gpp);
+        const int Yb = w.Ty + 2, passes = a.Cin / (8 * w.load);
         w.ngr = ((3 * w.gpp - 1) * Yb + 3 + 1) / 2 * 2;  // N is a multiple of 16
         w.ra = w.kst * 256;
         w.dslot = w.ns * (a.Cout / 8) * w.ra;
@@ -1451,7 +1467,7 @@ cudaError_t wgrad_launch(const WgradArgs& a, cudaStream_t st) {
     if (!wgrad_plan(a, sms, &wp, &wsmem) || !wgrad_ring_plan(a, sms, wp, &wr)) return cudaErrorInvalidValue;
     e = cudaFuncSetAttribute(k_wgrad_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, wr.smem);
     if (e != cudaSuccess) return e;
-    k_wgrad_ring<<<dim3((unsigned)wr.G, (unsigned)(a.Cin / (8 * wr.gpp))), 32 * kRingWarps, wr.smem, st>>>(a, wr);
+    k_wgrad_ring<<<dim3((unsigned)wr.G, (unsigned)(a.Cin / (8 * wr.load))), 32 * kRingWarps, wr.smem, st>>>(a, wr);
     return cudaGetLastError();
 }
 
@@ -1612,9 +1628,10 @@ extern "C" int sde_conv3d_wgrad_ring(int batch, int D, int H, int W, int Cin, in
         set_last_error("sde_conv3d_wgrad_ring: shape rejected by the weight gradient or without a plan");
         return SDE_EINVAL;
     }
-    const int32_t v[21] = {w.order, w.Ty,    w.gpp,   w.ngr, w.ns, w.nt,    w.kst,   w.P, w.ra,      w.drun,    w.dyx,
-                           w.xoff,  w.dslot, w.xslot, w.DS,  w.XS, w.x_off, w.items, w.G, w.copiers, w.arrivals};
-    for (int i = 0; i < n_fields && i < 21; ++i) fields[i] = v[i];
+    const int32_t v[23] = {w.order, w.Ty,    w.gpp,   w.ngr, w.ns, w.nt,    w.kst,   w.P, w.ra,      w.drun,    w.dyx,
+                           w.xoff,  w.dslot, w.xslot, w.DS,  w.XS, w.x_off, w.items, w.G, w.copiers, w.arrivals,
+                           w.load,  w.back};
+    for (int i = 0; i < n_fields && i < 23; ++i) fields[i] = v[i];
     if (smem_bytes) *smem_bytes = (uint64_t)w.smem;
     return SDE_OK;
 }

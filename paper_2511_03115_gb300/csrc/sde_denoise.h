@@ -105,7 +105,7 @@ struct WgradPlan {
 struct WgradRing {
     int order;         // 0: contiguous rows per CTA (short sums), 1: the row-block plan's items (long sums)
     int Ty, nyb;       // rows per item, H / Ty
-    int gpp;           // groups of eight input channels per pass
+    int gpp;           // groups of eight input channels in a plane slot
     int ngr;           // row groups of N (N = 8 ngr)
     int ns;            // copies of the dy row in M, shifted by s = -1..1 (3), 0..1 (2) or 0 (1)
     int nt;            // offsets at which the x window is read: 0 (1), -1..0 (2) or -1..1 (3)
@@ -121,6 +121,8 @@ struct WgradRing {
     int items;         // batch x nyb x D
     int G;             // CTAs per pass
     int copiers;       // copying warps that take part
+    int load;          // channel groups loaded per pass: gpp, or 1 (the others stay zero)
+    int back;          // positions by which the last K step's window starts before the step: it ends with the dy row
     int arrivals;      // arrivals per filling of a slot: 1 (every copier has a part of each), or all copiers
 };
 
