@@ -1431,8 +1431,13 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
         w.dslot = w.ns * (a.Cout / 8) * w.ra;
         w.xslot = w.gpp * Yb * w.P * 16;
         if (!order) {
-            w.G = sms / passes > 1 ? sms / passes : 1;  // all passes in one wave on the SMs
-            if (w.G > w.items) w.G = w.items;
+            // all passes in one wave on the SMs, or in as many as it takes for sums no longer than the
+            // row-block plan's: the error of an FP32 sum grows with its K steps, and narrow rows, whose
+            // K steps hold one row each, have up to three times as many of them
+            const int one = sms / passes > 1 ? sms / passes : 1;
+            const long long most = (long long)((wp.items + wp.G - 1) / wp.G) * wp.kst;
+            for (w.G = std::min(one, w.items); w.G < w.items; w.G = std::min(w.G + one, w.items))
+                if ((long long)((w.items + w.G - 1) / w.G) * w.kst <= most) break;
         }
         for (w.DS = kRingMaxD; w.DS >= 2; --w.DS)
             for (w.XS = order ? 3 * w.DS : kRingMaxX; w.XS >= (order ? 3 * w.DS : w.DS + 2); --w.XS) {
