@@ -834,17 +834,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 // with zeros there.  A row shorter than a K step has no earlier positions: its passes load one
 // group of channels, and the second group's part of each slot stays zero.
 //
-// One thread in each of warps 0-7 brings operands, its share of an item's 10 to 20 bulk copies; one
-// in each of warps 8-10 issues the MMAs of one offset t.  Each of these threads runs alone in its
-// warp at some seven cycles an instruction, so they keep positions, slots and phases by
-// increments: with the index divisions in their loops (three to four thousand cycles an item)
-// they, not the MMAs, set the time.  An item's commits release its dy slot and the planes no later
-// item needs.  A copying warp waits for a slot by the parity of its fillings, so no filling may go
-// by without it: in the long order only warps that copy a part of every item take part (without it
-// the item's MMAs cannot run), in the short order, where the planes' copies go round the warps, each of
-// them arrives for every filling.  dW stays in tensor memory over all of the CTA's items and is added to global memory
-// at the end, each CTA starting at another column (all walking the same order would meet on the
-// same addresses).
+// Warps 0-7 bring operands, their lanes an item's 10 to 38 bulk copies; warps 8-10 issue the MMAs of
+// one offset t each.  They run their loops as whole converged warps, with what one lane alone issues
+// predicated: branches for single lanes double the copying warps' time.  A warp issues at some seven
+// cycles an instruction, so they keep positions, slots and phases by increments: with the index
+// divisions in their loops (three to four thousand cycles an item) they, not the MMAs, set the time.
+// An item's commits release its dy slot and the planes no later item needs.  A copying warp waits
+// for a slot by the parity of its fillings, so no filling may go by without it: in the long order
+// only warps that copy a part of every item take part (without it the item's MMAs cannot run), in
+// the short order, where the planes' copies go round the warps, each of them arrives for every
+// filling.  dW stays in tensor memory over all of the CTA's items and is added to global memory at
+// the end, each CTA starting at another column (all walking the same order would meet on the same
+// addresses).
 //
 // Bound by the MMAs (N / 2 cycles each: the dense rate, a quarter of M used by 32 channels of the
 // long sums, three quarters of the short ones).  Before, one MMA a tap with 16 or 32 channels in N
@@ -967,86 +968,82 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
     const bool any = it.left > 0;
 
     if (warp < kRingCopyWarps) {
-        if (lane == 0 && warp < b.copiers) {
-            const Pcg pg{D, H, W};
-            const int gd = Cout >> 3, nd = b.ns * gd, gx = Cin >> 3;
-            const uint32_t xrun = (uint32_t)(Yb * b.P * 16);
-            // a dy run's copies: its whole K steps, and the last one's positions at that step's end
-            const uint32_t dmain = (uint32_t)(b.back ? (b.kst - 1) * 256 : b.drun), dtail = (uint32_t)b.drun - dmain;
-            const uint32_t tail_at = dmain + 16u * (uint32_t)b.back;
-            auto copy_dy = [&](uint32_t dst, const unsigned char* src, uint64_t* full) {
-                umma::bulk_g2s(dst, src, dmain, full);
-                if (dtail) umma::bulk_g2s(dst + tail_at, src + dmain, dtail, full);
-            };
-            const size_t plane = (size_t)(H + 2) * b.P * 16, vp = pg.vp() * 16;
-            // this warp's dy copies (copy i / gd of channel group i % gd; at most 16 in all) and the
-            // plane copies' sources, at z = y0 = n = 0
-            const unsigned char* dsrc[2];
-            uint32_t ddst[2];
-            bool mine[2];
-            for (int e = 0; e < 2; ++e) {
-                const int i = warp + kRingCopyWarps * e, s = i / gd, q = i - s * gd;
-                mine[e] = i < nd;
-                dsrc[e] = reinterpret_cast<const unsigned char*>(a.dy + 8 * pg.unit(0, gd, q, 0, 0, b.dyx - s));
-                ddst[e] = s_d + (uint32_t)(i * b.ra);
-            }
-            const unsigned char* xsrc =
-                reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.load, -1, -1, -1));
+        // Lanes 0-3 hold the warp's copies of dy rows (copy i = warp + 8 (lane / 2): channel group i % gd of
+        // shifted copy i / gd, at most 16 in all; even lanes the whole K steps, odd ones the last
+        // step's positions, which go to that step's end), lane 4 in the long order its plane copy (group
+        // warp % gpp of plane warp / gpp), and issue them with one instruction.  A lane that waits for a
+        // slot has a copy or an arrival in each of its fillings.
+        const Pcg pg{D, H, W};
+        const int gd = Cout >> 3, nd = b.ns * gd, gx = Cin >> 3;
+        const uint32_t xrun = (uint32_t)(Yb * b.P * 16);
+        const size_t plane = (size_t)(H + 2) * b.P * 16, vp = pg.vp() * 16;
+        const unsigned char* const xsrc =
+            reinterpret_cast<const unsigned char*>(a.x + 8 * pg.unit(0, gx, c * b.load, -1, -1, -1));
+        const unsigned char* src;  // at z = y0 = n = 0
+        uint32_t dst, bytes, slot_step;
+        size_t sample;
+        bool mine;
+        if (lane < 4) {
+            const int i = warp + kRingCopyWarps * (lane >> 1), s = i / gd, q = i - s * gd;
+            const uint32_t whole = (uint32_t)(b.back ? (b.kst - 1) * 256 : b.drun);
+            const bool rest = lane & 1;
+            mine = i < nd && (!rest || b.back);
+            src = reinterpret_cast<const unsigned char*>(a.dy + 8 * pg.unit(0, gd, q, 0, 0, b.dyx - s)) + (rest ? whole : 0u);
+            dst = s_d + (uint32_t)(i * b.ra) + (rest ? whole + 16u * (uint32_t)b.back : 0u);
+            bytes = rest ? (uint32_t)b.drun - whole : whole;
+            slot_step = (uint32_t)b.dslot;
+            sample = (size_t)gd * vp;
+        } else {
+            const int f = warp / b.gpp, q = warp - f * b.gpp;
+            mine = lane == 4 && b.order && f < 3;
+            src = xsrc + f * plane + q * vp;
+            dst = s_x + (uint32_t)(f * b.xslot) + (uint32_t)q * xrun;
+            bytes = xrun;
+            slot_step = 3u * (uint32_t)b.xslot;
+            sample = (size_t)gx * vp;
+        }
+        if (warp < b.copiers) {
             RingSlot sd;
-            int j = 0;
             bool ok = true;
-            if (b.order) {
-                // every item brings its three planes, on the dy slot's barrier; warp w's plane copy is
-                // group w % gpp of plane w / gpp
-                const int q = warp % b.gpp, f = warp / b.gpp;
-                const unsigned char* xs = xsrc + f * plane + q * vp;
-                const uint32_t xdst = s_x + (uint32_t)(f * b.xslot) + (uint32_t)q * xrun;
-                const uint32_t bytes = (uint32_t)(nd * b.drun) + 3u * (uint32_t)b.gpp * xrun;
-                for (; it.left > 0; ++j) {
-                    if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
+            if (b.order) {  // every item brings its three planes, on the dy slot's barrier
+                const uint32_t all = (uint32_t)(nd * b.drun) + 3u * (uint32_t)b.gpp * xrun;
+                for (int j = 0; it.left > 0; ++j) {
+                    if (j >= b.DS) ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag);
+                    if (!__all_sync(0xffffffffu, ok)) break;
                     uint64_t* full = &fulld[sd.i];
-                    const size_t at = (size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16);
-                    if (warp == 0) umma::mbar_arrive_expect_tx(full, bytes);
-                    if (f < 3)
-                        umma::bulk_g2s(xdst + (uint32_t)(3 * sd.i * b.xslot), xs + at + (size_t)it.n * gx * vp, xrun, full);
-#pragma unroll
-                    for (int e = 0; e < 2; ++e)
-                        if (mine[e])
-                            copy_dy(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp, full);
+                    umma::mbar_arrive_expect_tx_if(tid == 0, full, all);
+                    umma::bulk_g2s_if(mine, dst + (uint32_t)sd.i * slot_step,
+                                      src + ((size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16) + (size_t)it.n * sample),
+                                      bytes, full);
                     sd.advance(b.DS);
                     it.next(b, D);
                 }
             } else {
                 RingSlot sx;
-                int turn = nd, fresh = 3;  // fresh: planes this item brings; turn: copies go round the warps
-                size_t planes = 0;
-                for (; it.left > 0; ++j) {
-                    if (j >= b.DS && !(ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag))) break;
+                int turn = nd, fresh = 3, planes = 0;  // fresh: planes this item brings; turn: their copies go round the warps
+                const uint32_t dbytes = warp == 0 ? (uint32_t)(nd * b.drun) : 0u;
+                const uint32_t xbytes = warp == 0 ? (uint32_t)b.load * xrun : 0u;
+                const unsigned char* const xlane = xsrc + lane * vp;
+                const uint32_t xdst = s_x + (uint32_t)lane * xrun;
+                for (int j = 0; it.left > 0; ++j) {
+                    if (j >= b.DS) ok = pipe_wait(&emptyd[sd.i], sd.par ^ 1u, abort_flag);
+                    if (!__all_sync(0xffffffffu, ok)) break;
                     const size_t at = (size_t)it.z * plane + (size_t)it.yb * (b.P * 16);
-                    if (warp == 0)
-                        umma::mbar_arrive_expect_tx(&fulld[sd.i], (uint32_t)(nd * b.drun));
-                    else
-                        umma::mbar_arrive(&fulld[sd.i]);
-#pragma unroll
-                    for (int e = 0; e < 2; ++e)
-                        if (mine[e])
-                            copy_dy(ddst[e] + (uint32_t)(sd.i * b.dslot), dsrc[e] + at + (size_t)it.n * gd * vp,
-                                    &fulld[sd.i]);
-                    const unsigned char* xat = xsrc + at + (size_t)it.n * gx * vp + (3 - fresh) * plane;
+                    umma::mbar_arrive_expect_tx_if(lane == 0, &fulld[sd.i], dbytes);
+                    umma::bulk_g2s_if(mine, dst + (uint32_t)sd.i * slot_step, src + (at + (size_t)it.n * sample), bytes,
+                                      &fulld[sd.i]);
+                    const unsigned char* xat = xlane + (at + (size_t)it.n * gx * vp + (3 - fresh) * plane);
                     for (int f = 0; f < fresh; ++f, ++planes) {
-                        if (planes >= (size_t)b.XS && !(ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag))) break;
-                        if (warp == 0)
-                            umma::mbar_arrive_expect_tx(&fullx[sx.i], (uint32_t)b.load * xrun);
-                        else
-                            umma::mbar_arrive(&fullx[sx.i]);
-                        for (int q = 0; q < b.load; ++q, ++turn)
-                            if (turn % kRingCopyWarps == warp)
-                                umma::bulk_g2s(s_x + (uint32_t)(sx.i * b.xslot) + (uint32_t)q * xrun, xat + q * vp, xrun,
-                                               &fullx[sx.i]);
+                        if (planes >= b.XS) ok = pipe_wait(&emptyx[sx.i], sx.par ^ 1u, abort_flag);
+                        if (!__all_sync(0xffffffffu, ok)) break;
+                        umma::mbar_arrive_expect_tx_if(lane == 0, &fullx[sx.i], xbytes);
+                        umma::bulk_g2s_if(lane < b.load && (turn + lane) % kRingCopyWarps == warp,
+                                          xdst + (uint32_t)(sx.i * b.xslot), xat, xrun, &fullx[sx.i]);
+                        turn += b.load;
                         xat += plane;
                         sx.advance(b.XS);
                     }
-                    if (!ok) break;
+                    if (!__all_sync(0xffffffffu, ok)) break;
                     fresh = it.shares(b, D) ? 1 : 3;
                     sd.advance(b.DS);
                     it.next(b, D);

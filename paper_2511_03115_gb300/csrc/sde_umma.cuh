@@ -174,6 +174,22 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                  : "memory");
 }
 
+// mbar_arrive_expect_tx and bulk_g2s for the lanes of a converged warp that have one to issue.
+__device__ __forceinline__ void mbar_arrive_expect_tx_if(bool pred, uint64_t* m, uint32_t tx_bytes) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}\n" ::"r"(smem_addr(m)),
+        "r"(tx_bytes), "r"((uint32_t)pred)
+        : "memory");
+}
+__device__ __forceinline__ void bulk_g2s_if(bool pred, uint32_t dst, const void* src, uint32_t bytes, uint64_t* m) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+        "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}\n" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(smem_addr(m)), "r"((uint32_t)pred)
+        : "memory");
+}
+
 // Eight consecutive FP32 columns of this thread's tensor-memory lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     uint32_t r0, r1, r2, r3, r4, r5, r6, r7;
