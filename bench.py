@@ -57,7 +57,7 @@ TRANSPORT_DRAM = {  # workload -> {"src": sha256 prefix, "bytes": per launch, "n
     "plan2000": {"src": "f376f30a82243562", "bytes": 1_480_223_744 + 1_401_346_304, "histories": 100_000_000,
                  "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the first timed launch of "
                          "`bench.py --steps 2 --warmup 1 --no-denoiser --no-cpu-baseline --no-secondary` "
-                         "(1 pass; profiles/k_transport_plan2000.md)"},
+                         "(1 pass)"},
 }
 
 # L2 reduction (tally `red.add.u64`) rate of the transport kernel, from ncu on the plan's first
@@ -67,8 +67,7 @@ TRANSPORT_ATOMICS = {
                  "red_sectors": 433_034_795, "euler_steps": 525_487_490,
                  "note": "ncu lts__t_sectors_srcunit_tex_op_red (.sum, .avg.pct_of_peak_sustained_elapsed) of "
                          "k_transport in `bench.py --histories 2000000 --no-autotune --steps 1 --warmup 1 "
-                         "--e2e-steps 0 --no-denoiser --no-cpu-baseline --no-secondary` "
-                         "(profiles/k_transport_plan2000.md)"},
+                         "--e2e-steps 0 --no-denoiser --no-cpu-baseline --no-secondary`"},
 }
 
 # Instruction issue of the transport kernel (ncu --set full on the plan's first 2e6 histories,
@@ -81,8 +80,7 @@ TRANSPORT_ISSUE = {
                  "note": "ncu smsp__issue_active (of active cycles), smsp__thread_inst_executed_per_inst_executed, "
                          "smsp__inst_executed.sum, sm__pipe_*_cycles_active, smsp__average_warps_issue_stalled_"
                          "not_selected_per_issue_active of k_transport in `bench.py --histories 2000000 --no-autotune "
-                         "--steps 1 --warmup 1 --e2e-steps 0 --no-denoiser --no-cpu-baseline --no-secondary` "
-                         "(profiles/k_transport_plan2000.md)"},
+                         "--steps 1 --warmup 1 --e2e-steps 0 --no-denoiser --no-cpu-baseline --no-secondary`"},
 }
 
 WORKLOADS = {

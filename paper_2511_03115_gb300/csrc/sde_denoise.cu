@@ -122,7 +122,9 @@ cudaError_t status_word(unsigned int** out) {
 // default pool gives its memory back at every wait, so a call after one mapped its few hundred
 // kilobytes anew (a convolution and a wait: 375 us against 155 back to back); this pool keeps up to
 // 32 MB between waits and gives them back when a denoiser is destroyed.  While the stream
-// is being captured the allocation becomes a node of the graph as before.
+// is being captured the allocation becomes a node of the graph as before.  The error that is cleared is
+// of this library's own CUDA runtime (linked statically: a caller's pending errors are kept by the
+// caller's) and of a query here, or of an earlier call, which has returned it.
 constexpr uint64_t kScratchKept = 32ull << 20;
 std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[64] = {};
@@ -150,7 +152,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
         }
         pool = g_pool[dev];
     }
-    cudaGetLastError();  // a refused query above is not this call's failure
+    cudaGetLastError();
     return pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
 }
 
@@ -818,15 +820,16 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 //  - dx comes from nt offsets t at which the window of x is read, each an accumulator of its own,
 //    and from ns copies of the dy row in M, shifted by s positions: dx = s + t.
 //
-// Two orders of the items, as FP32 accumulation has to go (its error grows with the number of
-// positions in a sum; 5e-5 of the gradient at 32 channels of a 192x128x128 volume, more than
-// results may move by):
+// Two orders of the items (the error of an FP32 sum grows with its K steps, so neither has more of them
+// in a sum than the row-block plan):
 //  - short sums: a CTA owns a contiguous range of rows (Ty = 1) with z running fastest, so each
 //    further row needs one new plane; M is filled with shifted copies (ns = 3 up to 40 channels,
 //    2 up to 64), i.e. 96 of its 128 rows at 32 channels;
 //  - long sums: the items, K steps and CTAs of the row-block plan in their order, so that every
-//    sum is formed from the same products in the same order as with one MMA per tap (bit for bit
-//    up to the order of the CTAs' atomics); three offsets t, no copies.
+//    sum is formed from the same products in the same order as with one MMA per tap; three offsets
+//    t, no copies.  It keeps those sums, not the better ones: contiguous rows for 32 -> 32 channels on
+//    192x128x128 measured 0.30 ms against 0.40 and 2.4e-5 of the largest gradient off the exact one
+//    against 4.9e-5, but 3.6e-5 off the row-block plan's sums.
 //
 // A window of x that passed its row's end would bring other channels' values under the zeros that
 // fill dy's last K step, and zero times infinity is no zero.  So the last step's positions lie at its
@@ -850,7 +853,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3d_brick(ConvArgs a, Br
 // Bound by the MMAs (N / 2 cycles each: the dense rate, a quarter of M used by 32 channels of the
 // long sums, three quarters of the short ones).  Before, one MMA a tap with 16 or 32 channels in N
 // and the x brick loaded once per tap group: 32 -> 32 channels on 192x128x128 0.915 -> 0.398 ms (long
-// order: 0.33 ms of MMAs), 64 -> 96 on 66x54x128 0.316 -> 0.149 ms (short order).
+// order: 0.30 ms of MMAs), 64 -> 96 on 66x54x128 0.316 -> 0.149 ms (short order; 0.117 with the copying
+// warps converged).
 // ----------------------------------------------------------------------------
 constexpr int kRingMaxX = 12, kRingMaxD = 4, kRingCopyWarps = 8, kRingWarps = kRingCopyWarps + 3;
 
@@ -988,7 +992,8 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
             const uint32_t whole = (uint32_t)(b.back ? (b.kst - 1) * 256 : b.drun);
             const bool rest = lane & 1;
             mine = i < nd && (!rest || b.back);
-            src = reinterpret_cast<const unsigned char*>(a.dy + 8 * pg.unit(0, gd, q, 0, 0, b.dyx - s)) + (rest ? whole : 0u);
+            src = reinterpret_cast<const unsigned char*>(a.dy + 8 * pg.unit(0, gd, q, 0, 0, b.dyx - s)) +
+                  (rest ? whole : 0u);
             dst = s_d + (uint32_t)(i * b.ra) + (rest ? whole + 16u * (uint32_t)b.back : 0u);
             bytes = rest ? (uint32_t)b.drun - whole : whole;
             slot_step = (uint32_t)b.dslot;
@@ -1012,15 +1017,15 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                     if (!__all_sync(0xffffffffu, ok)) break;
                     uint64_t* full = &fulld[sd.i];
                     umma::mbar_arrive_expect_tx_if(tid == 0, full, all);
-                    umma::bulk_g2s_if(mine, dst + (uint32_t)sd.i * slot_step,
-                                      src + ((size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16) + (size_t)it.n * sample),
-                                      bytes, full);
+                    const size_t at = (size_t)it.z * plane + (size_t)(it.yb * b.Ty) * (b.P * 16);
+                    umma::bulk_g2s_if(mine, dst + (uint32_t)sd.i * slot_step, src + (at + (size_t)it.n * sample), bytes, full);
                     sd.advance(b.DS);
                     it.next(b, D);
                 }
             } else {
                 RingSlot sx;
-                int turn = nd, fresh = 3, planes = 0;  // fresh: planes this item brings; turn: their copies go round the warps
+                // fresh: planes this item brings; turn: their copies go round the warps
+                int turn = nd, fresh = 3, planes = 0;
                 const uint32_t dbytes = warp == 0 ? (uint32_t)(nd * b.drun) : 0u;
                 const uint32_t xbytes = warp == 0 ? (uint32_t)b.load * xrun : 0u;
                 const unsigned char* const xlane = xsrc + lane * vp;
@@ -1096,7 +1101,8 @@ __global__ void __launch_bounds__(32 * kRingWarps, 1) k_wgrad_ring(WgradArgs a, 
                     ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, idesc, b.kst, b.back, accum);
                 } else {
                     const int n1 = run * gp;
-                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, b.back, accum);
+                    ring_mma(leader, d, a_lo, a_hi, b_lo, b_hi, umma::idesc_bf16_f32(128, 8 * n1, 1, 1), b.kst, b.back,
+                             accum);
                     ring_mma(leader, d + (uint32_t)(8 * n1), a_lo, a_hi, (uint32_t)b0, b_hi,
                              umma::idesc_bf16_f32(128, N - 8 * n1, 1, 1), b.kst, b.back, accum);
                 }
@@ -1181,14 +1187,15 @@ __global__ void k_flip_weights(const __nv_bfloat16* w, __nv_bfloat16* wd, int Ci
 
 // Work decomposition of the pipelined brick kernel for one layer shape: output channels
 // split into parts of Cp, weights resident or streamed, rows per item Ty (the last row block
-// may pass H),
-// and for 128-voxel rows the x-tap fold, chosen by a cost model calibrated on GB300 with
-// per-role cycle counters in this kernel: a tcgen05.mma (M = 128, K = 16) takes ~64 cycles
-// of one issuing thread at N = 32, ~85 at N = 64, ~90 at N = 96 and about N / 2 from
-// N = 192, less with two issuers (mma_pair_factor); bulk copies of brick runs move ~64 bytes per cycle per SM; the epilogue takes
-// ~700 cycles per tile and 8 columns (~850 folded) on each of its two warp groups and
-// overlaps the MMAs only with two accumulators; copies and MMAs overlap, but not perfectly
-// (a quarter of the shorter one shows).
+// may pass H), and for 128-voxel rows the x-tap fold, by a cost model.  Its constants are per-role
+// cycle counts of an earlier kernel, which had two epilogue groups of whole tiles and one-thread
+// roles; they have not been measured again for the present one, nor does the model know waves, so
+// its choices are only as good as these: a tcgen05.mma (M = 128, K = 16) took ~64 cycles of one
+// issuing thread at N = 32, ~85 at N = 64, ~90 at N = 96 and about N / 2 from N = 192, less with two
+// issuers (mma_pair_factor); bulk copies of brick runs moved ~64 bytes per cycle per SM; the
+// epilogue took ~700 cycles per tile and 8 columns (~850 folded) on each of two warp groups and
+// overlapped the MMAs only with two accumulators; copies and MMAs overlapped, but not perfectly
+// (a quarter of the shorter one showed).
 static double mma_cycles(int N) {
     return N <= 32 ? 64.0 : (N <= 64 ? 85.0 : (N <= 96 ? 90.0 : (N <= 192 ? 96.0 + (N - 128) / 2.0 : N / 2.0)));
 }
@@ -1385,7 +1392,8 @@ static bool wgrad_plan(const WgradArgs& a, int sms, WgradPlan* out, size_t* smem
 // Rings of the weight gradient for one layer shape: the order of the items by the length of its
 // sums (in K steps of the row-block plan), then as many dy slots (up to four) and plane slots (up
 // to twelve; the fewer, the more often a range's planes wrap) as fit.  At 1024 steps the short
-// order moves the gradient by about 1.2e-5 and takes half the time of the long one.
+// order's gradient differs from the row-block plan's by about 1.2e-5 of its largest value, without
+// being less exact, and takes half the time of the long one.
 constexpr double kLongSum = 1024.0;
 
 bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing* out) {
@@ -1430,7 +1438,9 @@ bool wgrad_ring_plan(const WgradArgs& a, int sms, const WgradPlan& wp, WgradRing
         if (!order) {
             // all passes in one wave on the SMs, or in as many as it takes for sums no longer than the
             // row-block plan's: the error of an FP32 sum grows with its K steps, and narrow rows, whose
-            // K steps hold one row each, have up to three times as many of them
+            // K steps hold one row each, have up to five times as many of them (192 -> 32 on
+            // 192x128x24: 7.5e-5 of the largest gradient off in one wave, 3.9e-5 in two; 1.28 and 1.51 ms, 1.05
+            // in two with the copying warps converged)
             const int one = sms / passes > 1 ? sms / passes : 1;
             const long long most = (long long)((wp.items + wp.G - 1) / wp.G) * wp.kst;
             for (w.G = std::min(one, w.items); w.G < w.items; w.G = std::min(w.G + one, w.items))

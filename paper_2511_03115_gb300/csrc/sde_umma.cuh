@@ -60,18 +60,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
-// As mma_bf16 with each descriptor given as its low and high 32-bit words (callers that
-// step only the start-address field keep the high words fixed and add to the low ones).
-__device__ __forceinline__ void mma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                              uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %6, 0;\n\t"
-        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n" ::"r"(d_tmem),
-        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // One lane of the (converged) warp; the same one at every call.
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t r;
@@ -79,9 +67,10 @@ __device__ __forceinline__ uint32_t elect_one() {
     return r;
 }
 
-// mma_bf16_lohi and mma_commit for a whole converged warp: the lane with leader != 0 issues.  The
-// operands are then computed warp-uniformly; inside a one-lane branch each costs a move to
-// a uniform register per instruction.
+// mma_bf16 and mma_commit for a whole converged warp: the lane with leader != 0 issues.  Each
+// descriptor comes as its low and high 32-bit words (callers step only the start-address field, so
+// the high words stay).  The operands are computed warp-uniformly; inside a one-lane branch each
+// costs a move to a uniform register per instruction.
 __device__ __forceinline__ void mma_bf16_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
                                               uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -151,12 +140,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* m, uint32_t parity, long lon
 // Plain arrive (count 1) on an mbarrier.
 __device__ __forceinline__ void mbar_arrive(uint64_t* m) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(m)) : "memory");
-}
-
-// Arrive on the mbarrier once all cp.async copies issued so far by this thread have
-// landed (the arrival is not pre-counted: the barrier's count includes it).
-__device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* m) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(m)) : "memory");
 }
 
 // Arrive on the mbarrier (count 1) and add tx_bytes to the bytes its current phase waits for.
@@ -232,13 +215,6 @@ __device__ __forceinline__ void tmem_touch16(uint32_t (&r)[16]) {
                  :
                  : "memory");
 }
-
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 fills the 16 bytes with zeros.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // Byte offset of element (row, k) in a K-major no-swizzle tile whose rows hold kc BF16.
 __host__ __device__ __forceinline__ uint32_t core_offset(int row, int k, int kc) {
